@@ -112,6 +112,10 @@ struct Shape {
     static constexpr int B_BYTES = KSTEPS * ATOM_COL_BYTES;     // hi (or lo) of one stage
     static constexpr int BIMG_BYTES = 2 * B_BYTES;              // hi + lo
     static constexpr uint32_t SUM_COL = B_ROWS;
+    // Boundary of the accumulator's column halves: the same for tiles of every
+    // width, so that the low half of a tile never reaches into the high half of
+    // the tile before it, which may still be draining.
+    static constexpr int HALF = (B_ROWS / 2 + 15) & ~15;
     static_assert(B_ROWS % 16 == 0 && B_ROWS <= 208 && 2 * B_ROWS <= (int)A_COL,
                   "tile width within the tensor-memory budget");
     static_assert(BIMG_BYTES == tc_stage_bytes(NC, RD), "stage image size");
@@ -698,7 +702,7 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
             }
             const int cs = td.row0 >= I.mes_rows ? kp.chunk_stages_b : kp.chunk_stages;   // drain interval
             const int n_ch = (td.nst + cs - 1) / cs;
-            const int n_lo = n_real >= 32 ? ((n_real / 2 + 15) & ~15) : n_real;
+            const int n_lo = min(n_real, SH::HALF);
             for (int ch = 0; ch < n_ch && ok; ch++) {
                 for (int h = 0; h < 2; h++) {
                     const int c0 = h ? n_lo : 0, c1 = h ? n_real : n_lo;
@@ -802,7 +806,7 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
             const uint32_t idesc = idesc_f16(n_real, ELEM);
             const uint64_t bskip = (uint64_t)(td.cskip * (RD ? 32 : 64)) >> 4;
             // column halves [0, n_lo) and [n_lo, n_real) of the accumulator
-            const int n_lo = n_real >= 32 ? ((n_real / 2 + 15) & ~15) : n_real;
+            const int n_lo = min(n_real, SH::HALF);
             const int nh = n_real > n_lo ? 2 : 1;
             const uint32_t idesc_h[2] = {idesc_f16(n_lo, ELEM), nh == 2 ? idesc_f16(n_real - n_lo, ELEM) : 0u};
             int cs = 0;   // stage within the current accumulation chunk
