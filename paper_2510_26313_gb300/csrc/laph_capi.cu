@@ -64,6 +64,20 @@ constexpr int TC_DEFAULT_SUM = 8192;
 // Largest B-operand buffer of the tensor-core path: the timeslices of a batch
 // are processed in chunks whose stage images fit in it.
 constexpr size_t PSI_CAP_BYTES = 24ull << 30;
+// Cutting units into drains (see the plan's `emit`).  Work of a tile beside its
+// stages, in stages: a tile of one drain (16 stages) takes as long as 23 stages
+// of a long one (113 us for 7 tiles per CTA at L=24, N=32, 7 momenta, one
+// timeslice, against 0.7 us a stage).  Bytes moved in the time of a stage (about
+// 0.6 us at 4 TB/s).  The gain below which the tiles stay whole, the waves of
+// tiles above which a thin last wave no longer matters, and the most bytes of
+// extra partials.
+constexpr int TILE_STAGES = 8;
+constexpr double SPLIT_BYTES_PER_STAGE = 2.4e6;
+constexpr double SPLIT_MARGIN = 0.03;
+constexpr int SPLIT_MAX_WAVES = 10;
+constexpr size_t SPLIT_MAX_BYTES = 1ull << 30;
+// Jobs of the B-operand pass per SM below which jobs are made shorter.
+constexpr int PSI_JOBS_PER_SM = 8;
 
 }  // namespace
 
@@ -107,6 +121,8 @@ struct laph_plan {
     // tensor-core path: chunks of (instance, timeslice) units and their B-operand images
     laph::PsiUnit *d_units = nullptr;
     std::vector<laph::PsiUnit> h_units;
+    std::vector<TileDev> h_tiles;   // kept only when some unit is cut into drains (laph_plan_set_chunk_sites)
+    int psi_group = laph::TC_PSI_GROUP;   // stages per job of the B-operand pass
     // laph_plan_execute_host: copy streams and per-chunk events, made on first use
     cudaStream_t h2d = nullptr, d2h = nullptr;
     // tensor-core path: the FP64 site reduction of chunk c runs on `side`
@@ -119,7 +135,9 @@ struct laph_plan {
         int unit0, n_units;
         long long n_jobs;
         long long tile0, n_tiles;
-        long long n_red;   // blocks of the FP64 reduction
+        long long n_red;         // blocks of the FP64 reduction
+        int n_split;             // trailing units cut into drains
+        long long n_red_split;   // blocks of their reduction
     };
     std::vector<Chunk> chunks;
     // schedule of the tensor-core path: timeslices per chunk (0: chunks filled by
@@ -528,27 +546,36 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     // site block; order 0 runs them as (column tile, site block, row tile), so
     // that the tiles sharing one range of B stage images run side by side,
     // order 1 as (row tile, site block, column tile).
-    std::function<void(long long, int)> emit = [&](long long pc, int tile_order) {
+    // The last n_split units are cut into tiles of one drain interval (see
+    // PsiUnit::split).
+    auto drain_stages = [&]() { return std::max(1, p->chunk_sites * 3 / laph::TC_KSTAGE); };
+    auto emit_tables = [&](long long pc, int tile_order, int n_split) {
+        const int cs = drain_stages(), first_split = p->total_ts - n_split;
         tiles.clear();
         units.clear();
         p->chunks.clear();
         psi_max = part_max = 0;
-        laph_plan::Chunk cur{0, 0, 0, 0, 0, 0};
+        laph_plan::Chunk cur{};
         size_t cur_bytes = 0, cur_psi = 0;
         long long cur_part = 0;   // float2 entries of the chunk's partial buffer
         for (int n : order) {
             const InstDev &d = p->h_inst[n];
-            std::vector<TileDev> one;
-            if (!tc) {
-                one = ones[n];
-            } else {
+            const long long n_out = d.n_outB + d.n_outM;
+            // the tiles of one timeslice: one per site block, or one per drain interval
+            auto tiles_of = [&](bool split) {
+                if (!tc) return ones[n];
+                std::vector<TileDev> one;
                 for (const TileDev &u : ones[n])
                     for (int sc = 0; sc < d.n_sc; sc++) {
-                        TileDev v = u;
-                        v.s0 = sc * d.sc_stages;
-                        v.nst = std::min(d.sc_stages, d.n_st - v.s0);
-                        v.part_off = (long long)sc * (d.n_outB + d.n_outM);
-                        one.push_back(v);
+                        const int b0 = sc * d.sc_stages, b1 = std::min(b0 + d.sc_stages, d.n_st);
+                        const int step = split ? cs : b1 - b0, dps = split ? (d.sc_stages + cs - 1) / cs : 1;
+                        for (int s0 = b0; s0 < b1; s0 += step) {
+                            TileDev v = u;
+                            v.s0 = s0;
+                            v.nst = std::min(step, b1 - s0);
+                            v.part_off = ((long long)sc * dps + (s0 - b0) / step) * n_out;
+                            one.push_back(v);
+                        }
                     }
                 std::stable_sort(one.begin(), one.end(), [tile_order](const TileDev &x, const TileDev &y) {
                     const int xa = tile_order ? x.row0 : x.col0, ya = tile_order ? y.row0 : y.col0;
@@ -557,22 +584,38 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
                     if (x.s0 != y.s0) return x.s0 < y.s0;
                     return xb < yb;
                 });
-            }
+                return one;
+            };
+            std::vector<TileDev> one;
+            int one_split = -1;
             for (int t = 0; t < d.T; t++) {
+                const bool split = tc && (int)units.size() >= first_split;
+                if (one_split != (split ? 1 : 0)) {
+                    one = tiles_of(split);
+                    one_split = split ? 1 : 0;
+                }
                 if (tc) {
                     const bool full = pc > 0 ? cur.n_units >= pc : cur_bytes + unit_bytes[n] > psi_target;
                     if (cur.n_units > 0 && full) {
                         p->chunks.push_back(cur);
                         psi_max = std::max(psi_max, cur_psi);
                         part_max = std::max(part_max, (size_t)cur_part * sizeof(float2));
-                        cur = laph_plan::Chunk{(int)units.size(), 0, 0, (long long)tiles.size(), 0, 0};
+                        cur = laph_plan::Chunk{};
+                        cur.unit0 = (int)units.size();
+                        cur.tile0 = (long long)tiles.size();
                         cur_bytes = cur_psi = 0;
                         cur_part = 0;
                     }
-                    units.push_back(laph::PsiUnit{n, t, (long long)cur_psi, cur.n_jobs, cur_part, cur.n_red});
+                    units.push_back(laph::PsiUnit{n, t, split ? cs : 0, 0, (long long)cur_psi, cur.n_jobs, cur_part,
+                                                  split ? cur.n_red_split : cur.n_red});
                     cur.n_units++;
-                    cur.n_jobs += (long long)d.n_ct * ((d.n_st + laph::TC_PSI_GROUP - 1) / laph::TC_PSI_GROUP);
-                    cur.n_red += (d.n_outB + d.n_outM + laph::TC_RED_BLOCK - 1) / laph::TC_RED_BLOCK;
+                    cur.n_jobs += (long long)d.n_ct * ((d.n_st + p->psi_group - 1) / p->psi_group);
+                    if (split) {
+                        cur.n_split++;
+                        cur.n_red_split += (n_out + laph::TC_RED_BLOCK_SPLIT - 1) / laph::TC_RED_BLOCK_SPLIT;
+                    } else {
+                        cur.n_red += (n_out + laph::TC_RED_BLOCK - 1) / laph::TC_RED_BLOCK;
+                    }
                 }
                 for (TileDev u : one) {
                     u.t = t;
@@ -586,7 +629,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
                     cur.n_tiles += (long long)one.size();
                     cur_bytes += unit_bytes[n];
                     cur_psi += (size_t)d.n_ct * d.n_st * laph::tc_stage_bytes(p->tile_cols, p->rows2);
-                    cur_part += (long long)d.n_sc * (d.n_outB + d.n_outM);
+                    cur_part += (long long)d.n_sc * (split ? (d.sc_stages + cs - 1) / cs : 1) * n_out;
                 }
             }
         }
@@ -605,8 +648,78 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             }
         }
         p->h_units = units;
+        p->h_tiles.clear();
+        if (n_split > 0) p->h_tiles = tiles;
         p->sched_per_chunk = pc;
         p->sched_order = tile_order;
+    };
+    // Time of the last chunk's contraction, in K stages, when its last n_split
+    // units are cut into drains: whole tiles start in table order on the first
+    // CTA that is free, the short tiles of the cut units then fill the chip
+    // evenly.  A cut unit costs the traffic of its extra partials too (written and
+    // read once each, SPLIT_BYTES_PER_STAGE bytes in the time of a stage).
+    auto last_chunk_time = [&](int n_split, size_t *extra_bytes) -> double {
+        const int cs = drain_stages();
+        const laph_plan::Chunk &c = p->chunks.back();
+        std::vector<long long> free_at(sms, 0);   // a heap, earliest first
+        const auto later = std::greater<long long>();
+        long long end = 0, total = 0, longest = 0;
+        *extra_bytes = 0;
+        for (int u = 0; u < c.n_units; u++) {
+            const InstDev &d = p->h_inst[units[c.unit0 + u].inst];
+            const bool split = u >= c.n_units - n_split;
+            const long long pairs = (long long)ones[units[c.unit0 + u].inst].size();
+            for (int b0 = 0; b0 < d.n_st; b0 += d.sc_stages) {
+                const int st = std::min(d.sc_stages, d.n_st - b0), nd = split ? (st + cs - 1) / cs : 1;
+                total += pairs * (st + nd * TILE_STAGES);
+                if (split) {
+                    longest = std::max<long long>(longest, std::min(st, cs) + TILE_STAGES);
+                    *extra_bytes += (size_t)(nd - 1) * (size_t)(d.n_outB + d.n_outM) * sizeof(float2);
+                    continue;
+                }
+                for (long long q = 0; q < pairs; q++) {
+                    std::pop_heap(free_at.begin(), free_at.end(), later);
+                    free_at.back() += st + TILE_STAGES;
+                    end = std::max(end, free_at.back());
+                    std::push_heap(free_at.begin(), free_at.end(), later);
+                }
+            }
+        }
+        if (n_split) end = std::max(end, total / sms + longest);
+        return (double)end + 2.0 * (double)*extra_bytes / SPLIT_BYTES_PER_STAGE;
+    };
+    // The tables of a schedule, with as many trailing units of the last chunk
+    // cut into drains as pays: none of a batch that fills the chip anyway, all
+    // of a small one (one timeslice at L=24, N=32 is 18 tiles of up to 1024
+    // stages on 152 SMs), a few where the last wave of tiles is thin.  Units
+    // are cut only where both kinds of tile share one drain interval, within
+    // SPLIT_MAX_BYTES of extra partials.
+    std::function<void(long long, int)> emit = [&](long long pc, int tile_order) {
+        p->psi_group = laph::TC_PSI_GROUP;
+        emit_tables(pc, tile_order, 0);
+        if (!tc || p->chunks.empty()) return;
+        long long jobs = 0;
+        for (const laph_plan::Chunk &c : p->chunks) jobs = std::max(jobs, c.n_jobs);
+        // the B-operand pass walks a job's stages one after the other: shorter jobs until every SM has PSI_JOBS_PER_SM
+        while (p->psi_group > 1 && jobs < (long long)PSI_JOBS_PER_SM * sms) {
+            p->psi_group /= 2;
+            jobs *= 2;
+        }
+        const laph_plan::Chunk last = p->chunks.back();
+        int best = 0;
+        if ((p->chunk_sites_b == 0 || p->chunk_sites_b == p->chunk_sites) && last.n_tiles <= (long long)SPLIT_MAX_WAVES * sms) {
+            size_t extra = 0;
+            double best_t = last_chunk_time(0, &extra) * (1.0 - SPLIT_MARGIN);
+            for (int u = 1; u <= last.n_units; u = u < 4 || u == last.n_units ? u + 1 : std::min(2 * u, last.n_units)) {
+                const double t = last_chunk_time(u, &extra);
+                if (extra > SPLIT_MAX_BYTES) break;
+                if (t < best_t) {
+                    best = u;
+                    best_t = t;
+                }
+            }
+        }
+        if (best > 0 || p->psi_group != laph::TC_PSI_GROUP) emit_tables(pc, tile_order, best);
     };
     // device copies of the tables and the workspace layout (tensor-core modes:
     // per-timeslice max |phi| bits and one tile counter per chunk, both cleared
@@ -750,11 +863,68 @@ int laph_plan_sum_sites(const laph_plan *plan, int *sum_sites, int *max_site_blo
     return LAPH_OK;
 }
 
+// Takes back the cut into drains (its tiles and partials are made for one drain
+// interval): the unit's tiles cover whole site blocks again.  The workspace
+// layout stays; whole site blocks need a part of it.
+static int merge_drains(laph_plan *plan)
+{
+    if (plan->h_tiles.empty()) return LAPH_OK;
+    std::vector<TileDev> tiles;
+    std::vector<laph::PsiUnit> units = plan->h_units;
+    std::vector<laph_plan::Chunk> chunks = plan->chunks;
+    double flops = 0.0;
+    const int terms = (plan->mode == LAPH_MODE_TC_F16X3 || plan->mode == LAPH_MODE_TC_BF16X3) ? 3 : 1;
+    for (laph_plan::Chunk &c : chunks) {
+        const long long tile0 = (long long)tiles.size();
+        std::vector<long long> part(plan->total_ts, 0);
+        std::vector<int> split(plan->total_ts, 0);
+        c.n_red = c.n_red_split = 0;
+        c.n_split = 0;
+        for (int u = c.unit0; u < c.unit0 + c.n_units; u++) {
+            const InstDev &d = plan->h_inst[units[u].inst];
+            const long long n_out = d.n_outB + d.n_outM;
+            part[d.ts_base + units[u].t] = units[u].part_off;
+            split[d.ts_base + units[u].t] = units[u].split;
+            units[u].split = 0;
+            units[u].red0 = c.n_red;
+            c.n_red += (n_out + laph::TC_RED_BLOCK - 1) / laph::TC_RED_BLOCK;
+        }
+        for (long long q = c.tile0; q < c.tile0 + c.n_tiles; q++) {
+            TileDev v = plan->h_tiles[q];
+            const InstDev &d = plan->h_inst[v.inst];
+            const int ts = d.ts_base + v.t;
+            if (split[ts]) {
+                if (v.s0 % d.sc_stages) continue;
+                v.nst = std::min(d.sc_stages, d.n_st - v.s0);
+                v.part_off = part[ts] + (long long)(v.s0 / d.sc_stages) * (d.n_outB + d.n_outM);
+            }
+            const int n_real =
+                plan->rows2 ? ((v.ncols + 15) & ~15) - v.cskip : 2 * ((v.ncols + 7) & ~7) - 2 * v.cskip;
+            flops += 2.0 * laph::TC_TR * n_real * (2 * laph::TC_KSTAGE) * terms * v.nst;
+            tiles.push_back(v);
+        }
+        c.tile0 = tile0;
+        c.n_tiles = (long long)tiles.size() - tile0;
+    }
+    CK(cudaMemcpy(plan->d_tiles, tiles.data(), sizeof(TileDev) * tiles.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(plan->d_units, units.data(), sizeof(laph::PsiUnit) * units.size(), cudaMemcpyHostToDevice));
+    plan->h_units = units;
+    plan->chunks = chunks;
+    plan->n_tiles = (long long)tiles.size();
+    plan->mma_flops = flops;
+    plan->h_tiles.clear();
+    return LAPH_OK;
+}
+
 int laph_plan_set_chunk_sites(laph_plan *plan, int chunk_sites)
 {
     if (!plan || chunk_sites < 0 || chunk_sites > (1 << 24)) return LAPH_ERR_ARG;
     const bool tc = is_tc_mode(plan->mode);
     if (chunk_sites == 0) chunk_sites = tc ? TC_DEFAULT_CHUNK : SIMT_DEFAULT_CHUNK;
+    if (chunk_sites != plan->chunk_sites) {
+        const int rc = merge_drains(plan);
+        if (rc != LAPH_OK) return rc;
+    }
     plan->chunk_sites = chunk_sites;
     return LAPH_OK;
 }
@@ -811,7 +981,7 @@ static int launch_tc_chunk(laph_plan *p, char *ws, size_t ci, const laph::TcConf
     const laph_plan::Chunk &c = p->chunks[ci];
     const int ps = (int)(p->n_ptimed % laph_plan::RING), cs = (int)(p->n_timed % laph_plan::RING);
     if (timing) CK(cudaEventRecord(p->pv_begin[ps], s));
-    e = laph::launch_psi(p->d_inst, p->d_units + c.unit0, c.n_units, c.n_jobs, maxbits, cfg.elem, cfg.ncols, cfg.rows2,
+    e = laph::launch_psi(p->d_inst, p->d_units + c.unit0, c.n_units, c.n_jobs, p->psi_group, maxbits, cfg.elem, cfg.ncols, cfg.rows2,
                          psi, s);
     if (e != cudaSuccess) return cuda_fail(e, "psi");
     if (timing) {
@@ -831,7 +1001,8 @@ static int launch_tc_chunk(laph_plan *p, char *ws, size_t ci, const laph::TcConf
     CK(cudaEventRecord(p->ev_tc[ci], s));
     CK(cudaStreamWaitEvent(p->side, p->ev_tc[ci], 0));
     if (timing) CK(cudaEventRecord(p->rd_begin[cs], p->side));
-    e = laph::launch_reduce(p->d_inst, p->d_units + c.unit0, c.n_units, c.n_red, maxbits, part, p->side);
+    e = laph::launch_reduce(p->d_inst, p->d_units + c.unit0, c.n_units, c.n_split, c.n_red, c.n_red_split, maxbits, part,
+                            p->side);
     if (e != cudaSuccess) return cuda_fail(e, "site reduction");
     if (timing) CK(cudaEventRecord(p->rd_end[cs], p->side));
     CK(cudaEventRecord(p->ev_red[ci], p->side));
@@ -1267,7 +1438,9 @@ int laph_plan_launches_per_execute(const laph_plan *plan, int *n)
     const int ptr_launches = (plan->n_inst + 63) / 64;
     if (is_tc_mode(plan->mode))
         *n = ptr_launches + 2 * plan->n_inst /* scale, blockify */ +
-             3 * (int)plan->chunks.size() /* psi, contraction, FP64 site reduction */;
+             3 * (int)plan->chunks.size() /* psi, contraction, FP64 site reduction */ +
+             (!plan->chunks.empty() && plan->chunks.back().n_split > 0 &&
+              plan->chunks.back().n_split < plan->chunks.back().n_units) /* a reduction for either kind of unit */;
     else
         *n = ptr_launches + (int)((plan->n_tiles + 0x7ffffffeLL) / 0x7fffffffLL);
     return LAPH_OK;

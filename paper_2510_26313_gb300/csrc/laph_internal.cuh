@@ -92,9 +92,16 @@ struct TileDev {
 // Psi buffer; job0 is the index of its first (column tile, stage group) job
 // within the chunk.  Its FP32 partial sums occupy n_sc * (n_outB + n_outM)
 // float2 from part_off of the chunk's partial buffer; red0 is the index of
-// its first block of the FP64 reduction within the chunk.
+// its first block of the FP64 reduction within the chunk (among the units with
+// split = 0, or among those with split > 0, which come last).  split > 0: the
+// unit's site blocks are cut into tiles of one drain interval (`split` K
+// stages) each, and every drain's sums are a partial of their own
+// (ceil(sc_stages / split) per site block, the last site block's trailing
+// ones unused); the reduction then forms the FP32 running sums of a site
+// block itself, in the order in which a whole tile adds its drains.
 struct PsiUnit {
     int inst, t;
+    int split, pad;
     long long psi_off;
     long long job0;
     long long part_off;
@@ -104,11 +111,12 @@ struct PsiUnit {
 __host__ __device__ inline long long binom2(long long n) { return n * (n - 1) / 2; }
 __host__ __device__ inline long long binom3(long long n) { return n * (n - 1) * (n - 2) / 6; }
 
-// Pair index q = C(j,2) + i  ->  (i, j), i < j.
+// Pair index q = C(j,2) + i  ->  (i, j), i < j.  The square root only has to be
+// near: the two loops make j exact.
 __host__ __device__ inline void pair_of(long long q, int &i, int &j)
 {
 #ifdef __CUDA_ARCH__
-    int jj = (int)((1.0 + sqrt(1.0 + 8.0 * (double)q)) * 0.5);
+    int jj = (int)((1.f + sqrtf(1.f + 8.f * (float)q)) * 0.5f);
 #else
     int jj = (int)((1.0 + __builtin_sqrt(1.0 + 8.0 * (double)q)) * 0.5);
 #endif
@@ -208,21 +216,24 @@ constexpr int TC_TR_ROWS2 = 64;   // complex rows per tile in the row-doubled la
 // Tile widths with compiled kernels for each layout.
 bool tc_shape_supported(int ncols, int rows2);
 constexpr int TC_MAX_STAGED = 160;  // staged row vectors per tile
-constexpr int TC_PSI_GROUP = 16;    // stages per job of the B-operand pass
-// Psi stage images of a chunk: jobs [0, n_jobs) over the units [0, n_units).
-cudaError_t launch_psi(const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs,
+constexpr int TC_PSI_GROUP = 16;    // most stages per job of the B-operand pass
+// Psi stage images of a chunk: jobs [0, n_jobs) over the units [0, n_units), `group` stages each.
+cudaError_t launch_psi(const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs, int group,
                        const unsigned *d_maxbits, int elem, int ncols, int rows2, uint8_t *psi, cudaStream_t s);
 // counter: a zeroed word of device memory; persistent CTAs claim tiles with it.
 cudaError_t launch_tc(const InstDev *d_inst, const TileDev *d_tiles, long long n_tiles,
                       const unsigned *d_maxbits, const uint8_t *psi, float2 *part, unsigned *counter,
                       const TcConfig &cfg, int *d_status, cudaStream_t s);
-// Output entries handled by one block of the FP64 reduction.
+// Output entries handled by one block of the FP64 reduction (units with split = 0, units cut into drains).
 constexpr int TC_RED_BLOCK = 1024;
+constexpr int TC_RED_BLOCK_SPLIT = 256;
 // FP64 reduction of a chunk: every output entry of the units [0, n_units) is
 // the sum over its site blocks, in block order, of the FP32 partials, scaled
-// back and stored to the caller's complex128 outputs.
-cudaError_t launch_reduce(const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_blocks,
-                          const unsigned *d_maxbits, const float2 *part, cudaStream_t s);
+// back and stored to the caller's complex128 outputs.  The last n_split units
+// are cut into drains and take n_split_blocks blocks of a launch of their own
+// (their red0 counts from 0 again).
+cudaError_t launch_reduce(const InstDev *d_inst, const PsiUnit *d_units, int n_units, int n_split, long long n_blocks,
+                          long long n_split_blocks, const unsigned *d_maxbits, const float2 *part, cudaStream_t s);
 // Stages in the contraction's shared-memory ring for tiles staging up to
 // max_staged row vectors (0: none fits).
 int tc_ring_depth(int max_staged, int ncols, int rows2);

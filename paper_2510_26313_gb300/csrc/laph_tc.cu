@@ -689,17 +689,9 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
             const bool rvalid = gr < I.rows;
             const bool meson = gr < I.mes_rows;
             const bool trip = I.kind == INST_TRIPLETS;
+            const int q = gr - I.mes_rows;
             int pi_ = 0, pj = 0;
-            long long q = 0;
-            if (rvalid && !meson) {
-                q = gr - I.mes_rows;
-                if (trip) {
-                    pi_ = (int)(q / I.N);
-                    pj = (int)(q - (long long)pi_ * I.N);
-                } else {
-                    pair_of(q, pi_, pj);
-                }
-            }
+            if (rvalid && !meson && !trip) pair_of(q, pi_, pj);
             const int cs = td.row0 >= I.mes_rows ? kp.chunk_stages_b : kp.chunk_stages;   // drain interval
             const int n_ch = (td.nst + cs - 1) / cs;
             const int n_lo = min(n_real, SH::HALF);
@@ -737,54 +729,44 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
             // tile done: the FP32 sums of its site block go to the partial
             // buffer in the output order of one timeslice (B entries, then M
             // entries), still scaled; the FP64 reduction over site blocks
-            // scales them back
-            const int P = I.P, N = I.N;
-            const long long n_trip = I.n_trip;
-            float2 *part = kp.part + td.part_off;
+            // scales them back.  The entry moves by `step` from momentum to
+            // momentum and, past the last, to the next vector k; one division
+            // per block of columns.  (With one drain per tile the write is as
+            // long as the tile's MMAs when every entry is worked out afresh.)
+            const long long N = I.N;
+            const int P = I.P;
+            const bool tri = !meson && !trip;                 // packed i < j < k
+            const long long step = meson ? N * I.Nc : (trip ? N * N * N : I.n_trip);
+            const long long row_off = meson ? I.n_outB + (long long)gr * I.Nc : (trip ? q * N : q);   // q = i N + j
+            const int k_min = !rvalid ? 0x7fffffff : (tri ? pj + 1 : 0);                  // columns k >= k_min are outputs
+            float2 *part = kp.part + td.part_off + row_off;
             for (int b = 0; b * 16 < n_real; b++) {
                 if (N_EH > 1 && b % N_EH != eh) continue;
                 uint32_t v[16];
                 tmem_ld16(tmem + lane_base + SUM_COL + 16u * b, v);
+                constexpr int BC = RD ? 16 : 8;               // complex columns per block
+                const int cc0 = cskip + BC * b;
+                int k = (td.col0 + cc0) / P, p = td.col0 + cc0 - k * P;
+                long long e = p * step + (tri ? binom3(k) : k);
                 tmem_wait_ld();
-                if (RD) {
-                    // lane quadrants 0, 1 hold the real parts of the complex
-                    // rows, quadrants 2, 3 the imaginary parts: each writes its half
-#pragma unroll
-                    for (int u = 0; u < 16; u++) {
-                        const int cc = cskip + 16 * b + u;
-                        if (!rvalid || cc >= ncols) continue;
-                        const int col = td.col0 + cc;
-                        const int k = col / P, p = col - k * P;
-                        long long e;
-                        if (meson) {
-                            e = I.n_outB + ((long long)p * N + gr) * I.Nc + k;
-                        } else if (trip) {
-                            e = (((long long)p * N + pi_) * N + pj) * N + k;
-                        } else {
-                            if (k <= pj) continue;
-                            e = (long long)p * n_trip + binom3(k) + q;
-                        }
-                        reinterpret_cast<float *>(part + e)[quad >> 1] = __uint_as_float(v[u]);
+#pragma unroll(RD ? 16 : 1)
+                for (int u = 0; u < BC; u++) {
+                    if (cc0 + u < ncols && k >= k_min) {
+                        // row-doubled: lane quadrants 0, 1 hold the real parts of the complex rows, quadrants 2, 3
+                        // the imaginary parts, and each writes its half
+                        if (RD)
+                            reinterpret_cast<float *>(part + e)[quad >> 1] = __uint_as_float(v[u]);
+                        else
+                            part[e] = make_float2(__uint_as_float(v[(2 * u) & 15]), __uint_as_float(v[(2 * u + 1) & 15]));
                     }
-                    continue;
-                }
-#pragma unroll 1
-                for (int u = 0; u < 8; u++) {
-                    const int cc = cskip + 8 * b + u;
-                    if (!rvalid || cc >= ncols) continue;
-                    const int col = td.col0 + cc;
-                    const int k = col / P, p = col - k * P;
-                    long long e;
-                    if (meson) {
-                        e = I.n_outB + ((long long)p * N + gr) * I.Nc + k;   // [p][i][k], k < Nc
-                    } else if (trip) {
-                        e = (((long long)p * N + pi_) * N + pj) * N + k;    // dense [p][i][j][k]
-                    } else {
-                        if (k <= pj) continue;
-                        e = (long long)p * n_trip + binom3(k) + q;
+                    e += step;
+                    if (++p == P) {
+                        p = 0;
+                        e += (tri ? binom2(k) : 1) - P * step;
+                        k++;
                     }
-                    part[e] = make_float2(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1]));
                 }
+                __syncwarp();
             }
         }
     } else {
@@ -895,7 +877,7 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
 
 // ------------------------------------------------------------ B stage images
 
-// Job = (unit, column tile ct, group of TC_PSI_GROUP consecutive stages); the
+// Job = (unit, column tile ct, `group` consecutive stages; TC_PSI_GROUP, fewer where a launch has few jobs); the
 // unit is the last one whose job0 <= job.  Thread (cu = tid / 2, j = tid % 2)
 // takes tile column cu (complex column col0 + cu = k * P + p) and, for every
 // stage st of the group and k-step ks, the four K entries
@@ -908,7 +890,8 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
 // whole 32-byte rows.
 template <int ELEM, int NC, bool RD>
 __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__ insts, const PsiUnit *__restrict__ units,
-                                                     int n_units, long long n_jobs, const unsigned *__restrict__ maxbits,
+                                                     int n_units, long long n_jobs, int group,
+                                                     const unsigned *__restrict__ maxbits,
                                                      uint8_t *__restrict__ psi)
 {
     using SH = Shape<NC, RD>;
@@ -926,11 +909,11 @@ __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__
         const PsiUnit un = units[lo];
         const InstDev &I = insts[un.inst];
         const int n_st = I.n_st;
-        const int n_grp = (n_st + TC_PSI_GROUP - 1) / TC_PSI_GROUP;
+        const int n_grp = (n_st + group - 1) / group;
         const int jl = (int)(job - un.job0);
         const int ct = jl / n_grp;
-        const int st0 = (jl - ct * n_grp) * TC_PSI_GROUP;
-        const int st1 = min(st0 + TC_PSI_GROUP, n_st);
+        const int st0 = (jl - ct * n_grp) * group;
+        const int st1 = min(st0 + group, n_st);
         const int col0 = ct * NC;
         const bool valid = cu < min(NC, I.cols - col0);
         const int V = (int)I.V;
@@ -1018,17 +1001,57 @@ __device__ __forceinline__ double scale2(double v, int k)
     return v * pow2d(k);
 }
 
-// Block = TC_RED_BLOCK consecutive output entries of one (instance,
-// timeslice) unit; the unit is the last one whose red0 <= block.  Entry e of
-// the unit's output order (B entries [p][...] first, then M entries
-// [p][i][k]) is the FP64 sum over site blocks sc = 0, 1, ... of the FP32
-// partials part[part_off + sc * n_out + e], times 2^-3s (B) or 2^-2s (M), s
-// the timeslice's exponent, written as complex128 or, for complex64 outputs,
-// rounded once to FP32.  Each thread owns RED_PER_THREAD entries, TC_RED_BLOCK /
-// RED_PER_THREAD apart, and adds each entry's partials in block order.
+// Writes output entry e (B entries first, then M) of timeslice t.
+__device__ __forceinline__ void red_store(const InstDev &I, int t, long long e, int s, double re, double im)
+{
+    const long long nB = I.n_outB;
+    const bool b = e < nB;
+    void *base = b ? (void *)I.outB : (void *)I.outM;
+    const long long o = b ? (long long)t * nB + e : (long long)t * I.n_outM + (e - nB);
+    const int k = b ? -3 * s : -2 * s;
+    const double vr = scale2(re, k), vi = scale2(im, k);
+    if (I.out_c64)
+        reinterpret_cast<float2 *>(base)[o] = make_float2(__double2float_rn(vr), __double2float_rn(vi));
+    else
+        reinterpret_cast<double2 *>(base)[o] = make_double2(vr, vi);
+}
+
+// Block = consecutive output entries of one (instance, timeslice) unit
+// (TC_RED_BLOCK of them, TC_RED_BLOCK_SPLIT of a unit cut into drains); the
+// unit is the last one whose red0 <= block.  Entry e of the unit's output order
+// (B entries [p][...] first, then M entries [p][i][k]) is the FP64 sum over site
+// blocks sc = 0, 1, ... of the FP32 partials part[part_off + sc * n_out + e],
+// times 2^-3s (B) or 2^-2s (M), s the timeslice's exponent, written as
+// complex128 or, for complex64 outputs, rounded once to FP32.  Each thread owns
+// RED_PER_THREAD entries, TC_RED_BLOCK / RED_PER_THREAD apart, and adds each
+// entry's partials in block order.
+//
+// A unit cut into drains has one partial per drain.  A site block's FP32
+// running sum is formed here with the additions a whole tile's epilogue makes
+// (round to nearest, drain 0 first), so the outputs are the same bits either
+// way.  The additions of one entry are a serial chain, so a thread takes one
+// entry (more blocks in flight) and issues RED_BATCH loads ahead of it: small
+// outputs are bound by load latency (L=24, N=32, 7 momenta, one timeslice:
+// 41,720 entries x 108 drains, 36 MB, read by 163 blocks).
 constexpr int RED_THREADS = 256;
 constexpr int RED_PER_THREAD = TC_RED_BLOCK / RED_THREADS;
+constexpr int RED_BATCH = 16;
 static_assert(RED_PER_THREAD * RED_THREADS == TC_RED_BLOCK, "reduction block shape");
+static_assert(TC_RED_BLOCK_SPLIT == RED_THREADS, "one entry per thread of a split unit");
+
+// The unit of block blk: the last one whose red0 <= blk.
+__device__ __forceinline__ PsiUnit red_unit(const PsiUnit *__restrict__ units, int n_units, long long blk)
+{
+    int lo = 0, hi = n_units - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (units[mid].red0 <= blk)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return units[lo];
+}
 
 __global__ void __launch_bounds__(RED_THREADS) reduce_kernel(const InstDev *__restrict__ insts,
                                                              const PsiUnit *__restrict__ units, int n_units,
@@ -1036,17 +1059,9 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_kernel(const InstDev *__re
                                                              const float2 *__restrict__ part)
 {
     for (long long blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
-        int lo = 0, hi = n_units - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (units[mid].red0 <= blk)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        const PsiUnit un = units[lo];
+        const PsiUnit un = red_unit(units, n_units, blk);
         const InstDev &I = insts[un.inst];
-        const long long nB = I.n_outB, n_out = nB + I.n_outM;
+        const long long n_out = I.n_outB + I.n_outM;
         const long long e0 = (blk - un.red0) * TC_RED_BLOCK + threadIdx.x;
         const float2 *src = part + un.part_off;
         const int n_sc = I.n_sc;
@@ -1076,25 +1091,50 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_kernel(const InstDev *__re
 #pragma unroll
         for (int q = 0; q < RED_PER_THREAD; q++) {
             const long long e = e0 + q * RED_THREADS;
-            if (e >= n_out) continue;
-            long long o;
-            int k;
-            void *base;
-            if (e < nB) {
-                base = I.outB;
-                o = (long long)un.t * nB + e;
-                k = -3 * s;
-            } else {
-                base = I.outM;
-                o = (long long)un.t * I.n_outM + (e - nB);
-                k = -2 * s;
-            }
-            const double vr = scale2(re[q], k), vi = scale2(im[q], k);
-            if (I.out_c64)
-                reinterpret_cast<float2 *>(base)[o] = make_float2(__double2float_rn(vr), __double2float_rn(vi));
-            else
-                reinterpret_cast<double2 *>(base)[o] = make_double2(vr, vi);
+            if (e < n_out) red_store(I, un.t, e, s, re[q], im[q]);
         }
+    }
+}
+
+__global__ void __launch_bounds__(RED_THREADS) reduce_split_kernel(const InstDev *__restrict__ insts,
+                                                                   const PsiUnit *__restrict__ units, int n_units,
+                                                                   long long n_blocks,
+                                                                   const unsigned *__restrict__ maxbits,
+                                                                   const float2 *__restrict__ part)
+{
+    for (long long blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
+        const PsiUnit un = red_unit(units, n_units, blk);
+        const InstDev &I = insts[un.inst];
+        const long long n_out = I.n_outB + I.n_outM;
+        const long long e = (blk - un.red0) * TC_RED_BLOCK_SPLIT + threadIdx.x;
+        if (e >= n_out) continue;
+        const int dps = (I.sc_stages + un.split - 1) / un.split;   // partials kept per site block
+        double re = 0.0, im = 0.0;
+        for (int sc = 0; sc < I.n_sc; sc++) {
+            const int st = min(I.sc_stages, I.n_st - sc * I.sc_stages);
+            const int nd = (st + un.split - 1) / un.split;
+            const float2 *ps = part + un.part_off + (long long)sc * dps * n_out + e;
+            float2 sum = make_float2(0.f, 0.f);
+            for (int d0 = 0; d0 < nd; d0 += RED_BATCH) {
+                float2 v[RED_BATCH];
+#pragma unroll
+                for (int q = 0; q < RED_BATCH; q++)
+                    v[q] = d0 + q < nd ? __ldcs(ps + (long long)(d0 + q) * n_out) : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int q = 0; q < RED_BATCH; q++) {
+                    if (d0 + q >= nd) break;
+                    if (d0 + q == 0) {
+                        sum = v[q];
+                    } else {
+                        sum.x = __fadd_rn(v[q].x, sum.x);
+                        sum.y = __fadd_rn(v[q].y, sum.y);
+                    }
+                }
+            }
+            re = sc ? re + widen(sum.x) : widen(sum.x);
+            im = sc ? im + widen(sum.y) : widen(sum.y);
+        }
+        red_store(I, un.t, e, scale_exp(maxbits[I.ts_base + un.t]), re, im);
     }
 }
 
@@ -1142,12 +1182,12 @@ cudaError_t launch_one(const InstDev *d_inst, const TileDev *d_tiles, long long 
 
 template <int NC, bool RD>
 void psi_launch(int elem, unsigned grid, const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs,
-                const unsigned *d_maxbits, uint8_t *psi, cudaStream_t s)
+                int group, const unsigned *d_maxbits, uint8_t *psi, cudaStream_t s)
 {
     if (elem == 0)
-        psi_kernel<0, NC, RD><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, d_maxbits, psi);
+        psi_kernel<0, NC, RD><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
     else
-        psi_kernel<1, NC, RD><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, d_maxbits, psi);
+        psi_kernel<1, NC, RD><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
 }
 
 }  // namespace
@@ -1195,36 +1235,43 @@ cudaError_t launch_tc(const InstDev *d_inst, const TileDev *d_tiles, long long n
     return cudaErrorNotSupported;
 }
 
-cudaError_t launch_reduce(const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_blocks,
-                          const unsigned *d_maxbits, const float2 *part, cudaStream_t s)
+cudaError_t launch_reduce(const InstDev *d_inst, const PsiUnit *d_units, int n_units, int n_split, long long n_blocks,
+                          long long n_split_blocks, const unsigned *d_maxbits, const float2 *part, cudaStream_t s)
 {
-    if (n_blocks <= 0 || n_units <= 0) return cudaSuccess;
-    const long long grid = n_blocks < (1LL << 20) ? n_blocks : (1LL << 20);
-    reduce_kernel<<<(unsigned)grid, RED_THREADS, 0, s>>>(d_inst, d_units, n_units, n_blocks, d_maxbits, part);
+    const int n_whole = n_units - n_split;
+    if (n_whole > 0 && n_blocks > 0) {
+        const long long grid = n_blocks < (1LL << 20) ? n_blocks : (1LL << 20);
+        reduce_kernel<<<(unsigned)grid, RED_THREADS, 0, s>>>(d_inst, d_units, n_whole, n_blocks, d_maxbits, part);
+    }
+    if (n_split > 0 && n_split_blocks > 0) {
+        const long long grid = n_split_blocks < (1LL << 20) ? n_split_blocks : (1LL << 20);
+        reduce_split_kernel<<<(unsigned)grid, RED_THREADS, 0, s>>>(d_inst, d_units + n_whole, n_split, n_split_blocks,
+                                                                   d_maxbits, part);
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_psi(const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs,
+cudaError_t launch_psi(const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs, int group,
                        const unsigned *d_maxbits, int elem, int ncols, int rows2, uint8_t *psi, cudaStream_t s)
 {
     if (n_jobs <= 0 || n_units <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)(n_jobs < (1LL << 20) ? n_jobs : (1LL << 20));
     if (!rows2 && ncols == 104)
-        psi_launch<104, false>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<104, false>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (!rows2 && ncols == 96)
-        psi_launch<96, false>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<96, false>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (!rows2 && ncols == 80)
-        psi_launch<80, false>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<80, false>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (!rows2 && ncols == 64)
-        psi_launch<64, false>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<64, false>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (rows2 && ncols == 208)
-        psi_launch<208, true>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<208, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (rows2 && ncols == 192)
-        psi_launch<192, true>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<192, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (rows2 && ncols == 176)
-        psi_launch<176, true>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<176, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (rows2 && ncols == 128)
-        psi_launch<128, true>(elem, grid, d_inst, d_units, n_units, n_jobs, d_maxbits, psi, s);
+        psi_launch<128, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else
         return cudaErrorNotSupported;
     return cudaGetLastError();
