@@ -10,8 +10,21 @@
 // table skips tiles that lie wholly below the k > j triangle.  Per chunk of
 // 16 sites the block forms the A and Psi operands in shared memory and every
 // thread accumulates a 4x4 complex micro-tile in FP32.  Every chunk_sites
-// sites the FP32 partial sums are added in FP64 into the output, which each
-// element's owner thread alone reads and writes (first chunk stores).
+// sites (rounded up to 16) the FP32 partial sums are added in FP64 into the
+// output, which each element's owner thread alone reads and writes (first
+// chunk stores).
+//
+// Bound by FP32 issue.  A warp owns 32 rows x 16 columns; a lane reads two
+// consecutive rows (columns) with one 16-byte load, and the lanes of a load
+// read 8 (4) such pairs side by side, so that no load conflicts: four loads
+// per 64 multiply-adds.  A warp leaves out the 8-column groups that none of its
+// rows needs (k <= j everywhere), which the tile table's 64 x 64 steps cannot:
+// at N=32 and 7 momenta the tiles hold 1.86 times the needed products, the
+// groups 1.12 times.  The groups left out are spread over the four schedulers.
+// Two operand buffers, one barrier per chunk: while some warps form the next
+// chunk others multiply this one.  Two blocks per SM.  L=24, T=48, N=32, 7
+// momenta: 26.5 -> 23.8 ms.  (Packed fma.rn.f32x2 on operands stored
+// in the doubled form they need: 28.3 ms.  Three blocks per SM: 26 ms.)
 #include "laph_internal.cuh"
 
 namespace laph {
@@ -19,134 +32,158 @@ namespace laph {
 namespace {
 constexpr int KS = 16;               // sites per shared-memory chunk
 constexpr int KC = 3 * KS;           // complex K entries per chunk
-constexpr int APITCH = SIMT_TR + 2;  // float2 pitch, 16-byte aligned rows
-constexpr int BPITCH = SIMT_TC + 2;
+constexpr int DRAIN = 16;            // a drain interval is a multiple of this many sites
+constexpr int PITCH = SIMT_TR + 2;   // float2 per K entry, 16-byte aligned rows
 constexpr int NTHREADS = 256;
-static_assert(SIMT_TR == 64 && SIMT_TC == 64, "thread mapping assumes 64x64 tiles");
+constexpr int NPT = SIMT_TR * KS / NTHREADS;   // rows (and columns) of a site formed per thread
+static_assert(SIMT_TR == 64 && SIMT_TC == 64 && NPT == 4, "thread mapping assumes 64x64 tiles");
+
+// One chunk's multiply-adds of a lane: rows 2 lr + {0, 1} + 16 m, columns
+// 2 lc + {0, 1} + 8 n, column groups n >= N0 (As, Bs point at the lane's first).
+template <int N0>
+__device__ __forceinline__ void mac(float2 (&acc)[4][4], const float2 *__restrict__ As, const float2 *__restrict__ Bs)
+{
+#pragma unroll 2
+    for (int kk = 0; kk < KC; kk++) {
+        float2 a[4], b[4];
+#pragma unroll
+        for (int m = 0; m < 2; m++) {
+            const float4 t = *reinterpret_cast<const float4 *>(As + kk * PITCH + 16 * m);
+            a[2 * m] = make_float2(t.x, t.y);
+            a[2 * m + 1] = make_float2(t.z, t.w);
+        }
+#pragma unroll
+        for (int n = N0; n < 2; n++) {
+            const float4 t = *reinterpret_cast<const float4 *>(Bs + kk * PITCH + 8 * n);
+            b[2 * n] = make_float2(t.x, t.y);
+            b[2 * n + 1] = make_float2(t.z, t.w);
+        }
+#pragma unroll
+        for (int m = 0; m < 4; m++)
+#pragma unroll
+            for (int n = 2 * N0; n < 4; n++) {
+                acc[m][n].x = fmaf(a[m].x, b[n].x, acc[m][n].x);
+                acc[m][n].x = fmaf(-a[m].y, b[n].y, acc[m][n].x);
+                acc[m][n].y = fmaf(a[m].x, b[n].y, acc[m][n].y);
+                acc[m][n].y = fmaf(a[m].y, b[n].x, acc[m][n].y);
+            }
+    }
+}
 }  // namespace
 
 __global__ void __launch_bounds__(NTHREADS, 2)
 simt_kernel(const InstDev *__restrict__ insts, const TileDev *__restrict__ tiles, int chunk_sites)
 {
-    extern __shared__ __align__(16) float2 sm[];
-    float2 *As = sm;                 // [KC][APITCH]
-    float2 *Bs = sm + KC * APITCH;   // [KC][BPITCH]
+    extern __shared__ __align__(16) float2 sm[];   // two buffers of [A: KC][PITCH], [Psi: KC][PITCH]
 
     const TileDev tile = tiles[blockIdx.x];
-    const InstDev I = insts[tile.inst];
-    const int tid = threadIdx.x;
+    const InstDev &I = insts[tile.inst];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long V = I.V;
     const int N = I.N, P = I.P;
-    const float2 *__restrict__ phit = I.phi + (long long)tile.t * N * V * 3;
-    const float2 *__restrict__ ph = I.phase;
+    const float2 *__restrict__ phit = I.phi + (long long)tile.t * N * V * 3, *__restrict__ phase = I.phase;
 
-    // ---- operand-production mapping: site s, rows/cols tid/KS + 16*m
+    // ---- operand-production mapping: site s, rows/cols tid/KS + 32*m
     const int s = tid % KS;
-    int ai[4], aj[4], bk[4], bp[4];
+    // vectors of this thread's rows and columns (as element offsets / V): rows and columns past the tile's end are
+    // formed from vector 0 and never read back; aj < 0 marks a meson row
+    int ai[NPT], aj[NPT], bk[NPT], bp[NPT];
 #pragma unroll
-    for (int m = 0; m < 4; m++) {
-        const int r = tid / KS + 16 * m;
+    for (int m = 0; m < NPT; m++) {
+        const int r = tid / KS + (NTHREADS / KS) * m;
         const int g = tile.row0 + r;
-        if (g >= I.rows) {
-            ai[m] = -1;
-            aj[m] = -1;
-        } else if (g < I.mes_rows) {
+        ai[m] = bk[m] = bp[m] = 0;
+        aj[m] = -1;
+        if (g < I.mes_rows)
             ai[m] = g;
-            aj[m] = -1;
-        } else {
-            int i, j;
-            pair_of(g - I.mes_rows, i, j);
-            ai[m] = i;
-            aj[m] = j;
-        }
+        else if (g < I.rows)
+            pair_of(g - I.mes_rows, ai[m], aj[m]);
         const int col = tile.col0 + r;
-        if (col >= I.cols) {
-            bk[m] = -1;
-            bp[m] = 0;
-        } else {
+        if (col < I.cols) {
             bk[m] = col / P;
             bp[m] = col - bk[m] * P;
         }
     }
+    const long long Vs = I.Vs;
 
-    // ---- accumulation mapping: rows ty*4+m, cols tx*4+n
-    const int ty = tid / 16, tx = tid % 16;
+    // ---- accumulation mapping (see mac)
+    // Warps w and w + 4 share a scheduler: they get
+    // column groups two apart, turned from block to block, so that the
+    // groups left out (the leading ones) are spread over the schedulers.
+    const int wr = (warp >> 2) * 32, wc = ((warp + 2 * (warp >> 2) + blockIdx.x) & 3) * 16;
+    const int r0 = wr + 2 * (lane >> 2), c0 = wc + 2 * (lane & 3);
+    // first column group the warp's rows need (2: none)
+    int n0 = 0;
+    {
+        const int gw = tile.row0 + wr, cw = tile.col0 + wc;
+        if (gw >= I.rows || cw >= I.cols) {
+            n0 = 2;
+        } else if (gw >= I.mes_rows) {
+            int i, j;
+            pair_of(gw - I.mes_rows, i, j);   // the smallest j of the warp's rows
+            while (n0 < 2 && (cw + 8 * n0 + 7) / P <= j) n0++;
+        }
+    }
     float2 acc[4][4];
 #pragma unroll
     for (int m = 0; m < 4; m++)
 #pragma unroll
         for (int n = 0; n < 4; n++) acc[m][n] = make_float2(0.f, 0.f);
 
+    // chunk ch of the operands into buffer buf
+    auto form = [&](long long ch, int buf) {
+        float2 *As = sm + buf * 2 * KC * PITCH;
+        const long long x = ch * KS + s;
+#pragma unroll
+        for (int m = 0; m < NPT; m++) {
+            float2 *pa = As + 3 * s * PITCH + tid / KS + (NTHREADS / KS) * m, *pb = pa + KC * PITCH;
+            if (x >= V) {   // past the last site
+#pragma unroll
+                for (int c = 0; c < 3; c++) pa[c * PITCH] = pb[c * PITCH] = make_float2(0.f, 0.f);
+                continue;
+            }
+            const int i = ai[m], j = aj[m], k = bk[m], p = bp[m];
+            const float2 *pu = phit + ((long long)i * V + x) * 3, *pw = phit + ((long long)k * V + x) * 3;
+            const float2 u[3] = {__ldg(pu), __ldg(pu + 1), __ldg(pu + 2)};
+            const float2 w[3] = {__ldg(pw), __ldg(pw + 1), __ldg(pw + 2)};
+            const float2 ph = __ldg(phase + (long long)p * Vs + x);
+            if (j >= 0) {
+                const float2 *pv = phit + ((long long)j * V + x) * 3;
+                const float2 v[3] = {__ldg(pv), __ldg(pv + 1), __ldg(pv + 2)};
+#pragma unroll
+                for (int c = 0; c < 3; c++) pa[c * PITCH] = cross_c(u, v, c);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 3; c++) pa[c * PITCH] = conjf2(u[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) pb[c * PITCH] = cmulf(ph, w[c]);
+        }
+    };
+
     const long long nchunks = (V + KS - 1) / KS;
+    const int interval = (chunk_sites + DRAIN - 1) / DRAIN * DRAIN;
     int since = 0;
     bool first_drain = true;
+    form(0, 0);
+    __syncthreads();
 
     for (long long ch = 0; ch < nchunks; ch++) {
-        const long long x = ch * KS + s;
-        const bool xin = x < V;
-#pragma unroll
-        for (int m = 0; m < 4; m++) {
-            float2 o[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            if (xin && ai[m] >= 0) {
-                const float2 *u = phit + ((long long)ai[m] * V + x) * 3;
-                float2 uu[3] = {__ldg(u), __ldg(u + 1), __ldg(u + 2)};
-                if (aj[m] < 0) {
-#pragma unroll
-                    for (int c = 0; c < 3; c++) o[c] = conjf2(uu[c]);
-                } else {
-                    const float2 *v = phit + ((long long)aj[m] * V + x) * 3;
-                    float2 vv[3] = {__ldg(v), __ldg(v + 1), __ldg(v + 2)};
-#pragma unroll
-                    for (int c = 0; c < 3; c++) o[c] = cross_c(uu, vv, c);
-                }
-            }
-            const int r = tid / KS + 16 * m;
-#pragma unroll
-            for (int c = 0; c < 3; c++) As[(3 * s + c) * APITCH + r] = o[c];
-        }
-#pragma unroll
-        for (int m = 0; m < 4; m++) {
-            float2 o[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            if (xin && bk[m] >= 0) {
-                const float2 *w = phit + ((long long)bk[m] * V + x) * 3;
-                const float2 phv = __ldg(ph + (long long)bp[m] * I.Vs + x);
-#pragma unroll
-                for (int c = 0; c < 3; c++) o[c] = cmulf(phv, __ldg(w + c));
-            }
-            const int cl = tid / KS + 16 * m;
-#pragma unroll
-            for (int c = 0; c < 3; c++) Bs[(3 * s + c) * BPITCH + cl] = o[c];
-        }
-        __syncthreads();
-
-#pragma unroll 4
-        for (int kk = 0; kk < KC; kk++) {
-            const float4 a01 = *reinterpret_cast<const float4 *>(As + kk * APITCH + ty * 4);
-            const float4 a23 = *reinterpret_cast<const float4 *>(As + kk * APITCH + ty * 4 + 2);
-            const float4 b01 = *reinterpret_cast<const float4 *>(Bs + kk * BPITCH + tx * 4);
-            const float4 b23 = *reinterpret_cast<const float4 *>(Bs + kk * BPITCH + tx * 4 + 2);
-            const float2 a[4] = {make_float2(a01.x, a01.y), make_float2(a01.z, a01.w), make_float2(a23.x, a23.y),
-                                 make_float2(a23.z, a23.w)};
-            const float2 b[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
-                                 make_float2(b23.z, b23.w)};
-#pragma unroll
-            for (int m = 0; m < 4; m++)
-#pragma unroll
-                for (int n = 0; n < 4; n++) {
-                    acc[m][n].x = fmaf(a[m].x, b[n].x, acc[m][n].x);
-                    acc[m][n].x = fmaf(-a[m].y, b[n].y, acc[m][n].x);
-                    acc[m][n].y = fmaf(a[m].x, b[n].y, acc[m][n].y);
-                    acc[m][n].y = fmaf(a[m].y, b[n].x, acc[m][n].y);
-                }
-        }
+        const bool more = ch + 1 < nchunks;
+        if (more) form(ch + 1, (int)(ch + 1) & 1);
+        const float2 *As = sm + (int)(ch & 1) * 2 * KC * PITCH + r0, *Bs = As - r0 + KC * PITCH + c0;
+        if (n0 == 0)
+            mac<0>(acc, As, Bs);
+        else if (n0 == 1)
+            mac<1>(acc, As, Bs);
         __syncthreads();
 
         since += KS;
-        if (since >= chunk_sites || ch == nchunks - 1) {
+        if (since >= interval || !more) {
             // ---- FP64 reduction of this chunk's partial sums into the output
 #pragma unroll
             for (int m = 0; m < 4; m++) {
-                const int g = tile.row0 + ty * 4 + m;
+                const int g = tile.row0 + r0 + (m & 1) + 16 * (m >> 1);
                 if (g >= I.rows) continue;
                 const bool meson = g < I.mes_rows;
                 int pi = 0, pj = 0;
@@ -157,7 +194,7 @@ simt_kernel(const InstDev *__restrict__ insts, const TileDev *__restrict__ tiles
                 }
 #pragma unroll
                 for (int n = 0; n < 4; n++) {
-                    const int col = tile.col0 + tx * 4 + n;
+                    const int col = tile.col0 + c0 + (n & 1) + 8 * (n >> 1);
                     if (col >= I.cols) continue;
                     const int k = col / P, p = col - k * P;
                     double2 *dst;
@@ -167,13 +204,13 @@ simt_kernel(const InstDev *__restrict__ insts, const TileDev *__restrict__ tiles
                         if (k <= pj) continue;
                         dst = I.outB + ((long long)tile.t * P + p) * I.n_trip + binom3(k) + q;
                     }
-                    double2 v = make_double2((double)acc[m][n].x, (double)acc[m][n].y);
+                    double2 d = make_double2((double)acc[m][n].x, (double)acc[m][n].y);
                     if (!first_drain) {
                         const double2 old = *dst;
-                        v.x += old.x;
-                        v.y += old.y;
+                        d.x += old.x;
+                        d.y += old.y;
                     }
-                    *dst = v;
+                    *dst = d;
                 }
             }
 #pragma unroll
@@ -191,7 +228,7 @@ cudaError_t launch_simt(const InstDev *d_inst, const TileDev *d_tiles, long long
 {
     (void)d_status;
     if (n_tiles <= 0) return cudaSuccess;
-    const size_t smem = (size_t)KC * (APITCH + BPITCH) * sizeof(float2);
+    const size_t smem = (size_t)4 * KC * PITCH * sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int chunk = cfg.chunk_sites > 0 ? cfg.chunk_sites : 1024;
