@@ -307,10 +307,12 @@ typedef struct {
     int sum_sites;   /* tensor-core modes: sites per block of the FP64 site reduction (default 8192, rounded down
                         to a multiple of 8): a tile covers one block, its running sums become one FP32 partial per
                         output, and the partials of all blocks are added in FP64 in block order */
-    int tile_cols;   /* tensor-core modes: complex columns per tile: 104 (default), 96, 80 or 64 in layout 0;
-                        176 (default), 192, 208 or 128 in layout 1 */
+    int tile_cols;   /* tensor-core modes: complex columns per tile: 104, 96, 80 or 64 in layout 0; 176 (default),
+                        192, 208 or 128 in layout 1.  0 with layout 0: the plan takes the shape (either layout) with the
+                        lowest estimated time, 104 or 96 columns of layout 0 for small problems; every shape gives
+                        the same results */
     int layout;      /* tensor-core modes: how the complex product is laid out on the real tensor cores.
-                        0 (default): every complex column of the phased operand is two real rows (re, im) of the
+                        0: every complex column of the phased operand is two real rows (re, im) of the
                         MMA's B operand, 128 complex rows per tile; 1: every complex row of the diquark / meson
                         operand is two real rows of the MMA's A operand (tensor-memory lanes r, 64+r), 64 complex
                         rows per tile, and the phased operand's stage images are half as large */

@@ -76,6 +76,16 @@ constexpr double SPLIT_BYTES_PER_STAGE = 2.4e6;
 constexpr double SPLIT_MARGIN = 0.03;
 constexpr int SPLIT_MAX_WAVES = 10;
 constexpr size_t SPLIT_MAX_BYTES = 1ull << 30;
+// Estimates for the choice of the tile shape (see the plan's `shape_us`), fitted
+// to the triplets at L=32, N=64, 19 momenta (us per stage of a long tile, 208 /
+// 192 / 128 accumulator columns in layout 0: 0.734 / 0.695 / 0.625;
+// layout 1, 208 / 176 / 128 columns: 0.747 / 0.698 / 0.636) and to the B-operand
+// pass (bytes written and read per us).
+constexpr double STAGE_US = 0.45, STAGE_US_COL = 0.00137;
+constexpr double RING_COST = 1.11;
+constexpr double PSI_BYTES_US = 6.3e6, PSI_BYTES_US_ROWS2 = 5.3e6;
+constexpr double SHAPE_MARGIN = 0.03;
+constexpr int SHAPE_MIN_STAGES = 16;   // per SM
 // Jobs of the B-operand pass per SM below which jobs are made shorter.
 constexpr int PSI_JOBS_PER_SM = 8;
 
@@ -430,39 +440,42 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             d.n_ct = (d.cols + TC - 1) / TC;
             std::vector<TileDev> &one = ones[n];
             one.clear();
+            const bool trip = d.kind == laph::INST_TRIPLETS;
+            // per row tile: the smallest j of a baryon row tile (rows of pairs i < j need only columns k > j; -1:
+            // every column) and the contiguous range of vectors its rows use (for triplets: of phi_u, and
+            // [w_lo, w_hi] of phi_v)
+            struct RowTile {
+                int jmin, v_lo, v_hi, w_lo, w_hi;
+            };
+            std::vector<RowTile> rts;
+            for (int row0 = 0; row0 < d.rows; row0 += TR) {
+                RowTile r{-1, d.N, -1, d.N, -1};
+                for (int g = row0; g < std::min(row0 + TR, d.rows); g++) {
+                    int i = g, j = g;
+                    if (g >= d.mes_rows && trip) {
+                        const int q = g - d.mes_rows;
+                        i = q / d.N;
+                        j = q - i * d.N;
+                        r.w_lo = std::min(r.w_lo, j);
+                        r.w_hi = std::max(r.w_hi, j);
+                        j = i;
+                    } else if (g >= d.mes_rows) {
+                        laph::pair_of(g - d.mes_rows, i, j);
+                        if (g == row0) r.jmin = j;
+                    }
+                    r.v_lo = std::min(r.v_lo, i);
+                    r.v_hi = std::max(r.v_hi, j);
+                }
+                rts.push_back(r);
+            }
             for (int col0 = 0; col0 < d.cols; col0 += TC) {
                 const int nc = std::min(TC, d.cols - col0);
                 const int kmin = col0 / d.P, kmax = (col0 + nc - 1) / d.P;
-                const bool trip = d.kind == laph::INST_TRIPLETS;
                 for (int row0 = 0; row0 < d.rows; row0 += TR) {
-                    // baryon blocks: rows of pairs i < j need only columns k > j
-                    int jmin = -1;
-                    if (row0 >= d.mes_rows && !trip) {
-                        int i, j;
-                        laph::pair_of(row0 - d.mes_rows, i, j);
-                        jmin = j;
-                    }
+                    const RowTile &rt = rts[row0 / TR];
+                    const int jmin = rt.jmin, v_lo = rt.v_lo, v_hi = rt.v_hi, w_hi = rt.w_hi;
+                    int w_lo = rt.w_lo;
                     if (jmin >= 0 && kmax <= jmin) continue;
-                    // contiguous range of vectors used by the rows of this tile (for
-                    // triplets: of phi_u, and [w_lo, w_hi] of phi_v)
-                    int v_lo = d.N, v_hi = -1, w_lo = d.N, w_hi = -1;
-                    for (int g = row0; g < std::min(row0 + TR, d.rows); g++) {
-                        if (g < d.mes_rows) {
-                            v_lo = std::min(v_lo, g);
-                            v_hi = std::max(v_hi, g);
-                        } else if (trip) {
-                            const int q = g - d.mes_rows, i = q / d.N, j = q - i * d.N;
-                            v_lo = std::min(v_lo, i);
-                            v_hi = std::max(v_hi, i);
-                            w_lo = std::min(w_lo, j);
-                            w_hi = std::max(w_hi, j);
-                        } else {
-                            int i, j;
-                            laph::pair_of(g - d.mes_rows, i, j);
-                            v_lo = std::min(v_lo, i);
-                            v_hi = std::max(v_hi, j);
-                        }
-                    }
                     const int nv = v_hi - v_lo + 1;
                     const int nw = trip ? w_hi - w_lo + 1 : 0;
                     if (!trip) w_lo = 0;
@@ -786,15 +799,77 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     const int opt_cols = opts ? opts->tile_cols : 0, opt_layout = opts ? opts->layout : 0;
     laph::Sched def{opt_cols ? opt_cols : (opt_layout ? 176 : laph::TC_TC),
                     opt_sum ? opt_sum : TC_DEFAULT_SUM, p->chunk_sites, -1, 0, opt_layout, opt_chunk_b};
-    PCK(apply(def));
-    // the default width is the widest whose stage ring stays 4 deep for the
-    // plan's row vectors (the staged vectors depend on the row tiles only):
-    // a shallower ring costs more than the wider tile gains
-    if (tc && !opt_cols && !opt_layout && laph::tc_ring_depth(p->max_staged, def.tile_cols, 0) < 4 &&
-        laph::tc_ring_depth(p->max_staged, 96, 0) > laph::tc_ring_depth(p->max_staged, def.tile_cols, 0)) {
-        def.tile_cols = 96;
-        PCK(apply(def));
+    // Estimated time (us) of an execute's B-operand pass and contraction with
+    // tiles of nc columns in layout r2.  A stage of a tile costs STAGE_US +
+    // STAGE_US_COL per accumulator column (both layouts); whole tiles on the
+    // first free CTA where there are few waves of them, else (or where the last
+    // wave can be cut into drains) spread evenly.  A stage ring of fewer than
+    // four buffers costs RING_COST.
+    auto shape_us = [&](int nc, int r2) -> double {
+        build_tiles(nc, r2);
+        set_sum(def.sum_sites);
+        const int ring = laph::tc_ring_depth(p->max_staged, nc, r2);
+        if (p->max_staged > laph::TC_MAX_STAGED || !ring) return 1e300;
+        double total = 0.0, bytes = 0.0;
+        long long n_tiles = 0;
+        auto stage_us = [&](const TileDev &u) {
+            const int n_real = r2 ? ((u.ncols + 15) & ~15) - u.cskip : 2 * ((u.ncols + 7) & ~7) - 2 * u.cskip;
+            return STAGE_US + STAGE_US_COL * n_real;
+        };
+        for (int n = 0; n < n_inst; n++) {
+            const InstDev &d = p->h_inst[n];
+            for (const TileDev &u : ones[n]) total += stage_us(u) * d.n_st * d.T;
+            n_tiles += (long long)ones[n].size() * d.n_sc * d.T;
+            bytes += (double)d.T * ((double)d.n_ct * d.n_st * laph::tc_stage_bytes(nc, r2) + 24.0 * d.Nc * d.V);
+        }
+        double us = total / sms;
+        if (n_tiles <= (long long)SPLIT_MAX_WAVES * sms) {
+            std::vector<double> free_at(sms, 0.0);
+            const auto later = std::greater<double>();
+            double end = 0.0;
+            for (int n = 0; n < n_inst; n++) {
+                const InstDev &d = p->h_inst[n];
+                for (int t = 0; t < d.T; t++)
+                    for (const TileDev &u : ones[n])
+                        for (int b0 = 0; b0 < d.n_st; b0 += d.sc_stages) {
+                            std::pop_heap(free_at.begin(), free_at.end(), later);
+                            free_at.back() += stage_us(u) * (std::min(d.sc_stages, d.n_st - b0) + TILE_STAGES);
+                            end = std::max(end, free_at.back());
+                            std::push_heap(free_at.begin(), free_at.end(), later);
+                        }
+            }
+            us = std::min(end, n_tiles >= 2 * sms ? 1.04 * us : (1.0 + TILE_STAGES / 16.0) * us);
+        }
+        return us * (ring < 4 ? RING_COST : 1.0) + bytes / (r2 ? PSI_BYTES_US_ROWS2 : PSI_BYTES_US);
+    };
+    // The default shape is 104 columns of layout 0, or 96 where the row vectors
+    // a tile stages would leave its ring shallower than four buffers.  A plan
+    // with enough work takes another shape where the estimate is better by
+    // SHAPE_MARGIN: layout 1 has half the B-operand bytes and 64-row tiles
+    // (meson rows alone fill half of a 128-row tile), a narrower tile of layout 0
+    // may cover the columns in as many tiles.  Every shape gives the same bits.
+    if (tc && !opt_cols && !opt_layout) {
+        const double us104 = shape_us(def.tile_cols, 0);
+        if (laph::tc_ring_depth(p->max_staged, def.tile_cols, 0) < 4 &&
+            laph::tc_ring_depth(p->max_staged, 96, 0) > laph::tc_ring_depth(p->max_staged, def.tile_cols, 0))
+            def.tile_cols = 96;
+        long long stages = 0;
+        for (int n = 0; n < n_inst; n++)
+            stages += (long long)ones[n].size() * p->h_inst[n].n_st * p->h_inst[n].T;
+        if (stages >= (long long)SHAPE_MIN_STAGES * sms) {
+            double best = (def.tile_cols == 96 ? shape_us(96, 0) : us104) * (1.0 - SHAPE_MARGIN);
+            const std::pair<int, int> shapes[] = {{96, 0}, {80, 0}, {64, 0}, {208, 1}, {176, 1}, {128, 1}};
+            for (const auto &sh : shapes) {
+                const double us = shape_us(sh.first, sh.second);
+                if (us < best) {
+                    best = us;
+                    def.tile_cols = sh.first;
+                    def.rows2 = sh.second;
+                }
+            }
+        }
     }
+    PCK(apply(def));
     if (tc && p->max_staged > laph::TC_MAX_STAGED) {
         free_plan(p);
         return LAPH_ERR_UNSUPPORTED;
