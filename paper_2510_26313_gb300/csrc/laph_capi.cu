@@ -1084,22 +1084,21 @@ static int launch_tc_chunk(laph_plan *p, char *ws, size_t ci, const laph::TcConf
     return LAPH_OK;
 }
 
-// Scale and site-blocked copy of the timeslices of chunk ci, one launch pair
-// per run of consecutive timeslices of one instance.
-static int launch_chunk_prep(laph_plan *p, char *ws, size_t ci, cudaStream_t s)
+// Scale and site-blocked copy of the units [unit0, unit0 + n_units): one launch each.
+static int launch_prep(laph_plan *p, char *ws, int unit0, int n_units, cudaStream_t s)
 {
     unsigned *maxbits = (unsigned *)(ws + p->off_maxbits);
-    const laph_plan::Chunk &c = p->chunks[ci];
-    for (int u = c.unit0; u < c.unit0 + c.n_units;) {
-        const int n = p->h_units[u].inst, t0 = p->h_units[u].t;
-        int nt = 1;
-        while (u + nt < c.unit0 + c.n_units && p->h_units[u + nt].inst == n && p->h_units[u + nt].t == t0 + nt) nt++;
-        cudaError_t e = laph::launch_scale_max_range(p->d_inst, n, t0, nt, p->phi_elems[n] / p->h_T[n], maxbits, s,
-                                                     p->h_inst[n].n_fields);
-        if (e == cudaSuccess) e = laph::launch_blockify_range(p->d_inst, n, p->h_inst[n], t0, nt, maxbits, s);
-        if (e != cudaSuccess) return cuda_fail(e, "scale/blockify");
-        u += nt;
+    long long elems = 1;
+    int nblk = 1;
+    for (int n = 0; n < p->n_inst; n++) {
+        elems = std::max(elems, p->phi_elems[n] / p->h_T[n]);
+        nblk = std::max(nblk, p->h_inst[n].nblk);
     }
+    const InstDev &d = p->h_inst[0];   // the kind of instance is the plan's
+    cudaError_t e = laph::launch_scale_max(p->d_inst, p->d_units + unit0, n_units, d.n_fields, elems, maxbits, s);
+    if (e != cudaSuccess) return cuda_fail(e, "scale_max");
+    e = laph::launch_blockify(p->d_inst, p->d_units + unit0, n_units, nblk, d.kind == laph::INST_TRIPLETS, maxbits, s);
+    if (e != cudaSuccess) return cuda_fail(e, "blockify");
     return LAPH_OK;
 }
 
@@ -1110,21 +1109,9 @@ static int launch_batch(laph_plan *p, void *workspace, cudaStream_t s)
     if (is_tc_mode(p->mode)) {
         if (!workspace || ((uintptr_t)workspace) % 256) return LAPH_ERR_WORKSPACE;
         char *ws = (char *)workspace;
-        unsigned *maxbits = (unsigned *)(ws + p->off_maxbits);
         CK(cudaMemsetAsync(ws, 0, p->ws_zero_bytes, s));
-        std::vector<long long> elems(p->n_inst);
-        std::vector<int> nf(p->n_inst);
-        for (int n = 0; n < p->n_inst; n++) {
-            elems[n] = p->phi_elems[n] / p->h_T[n];
-            nf[n] = p->h_inst[n].n_fields;
-        }
-        e = laph::launch_scale_max(p->d_inst, p->n_inst, p->h_ts_base.data(), p->h_T.data(), elems.data(), maxbits, s,
-                                   nf.data());
-        if (e != cudaSuccess) return cuda_fail(e, "scale_max");
-        for (int n = 0; n < p->n_inst; n++) {
-            e = laph::launch_blockify(p->d_inst, n, p->h_inst[n], maxbits, s);
-            if (e != cudaSuccess) return cuda_fail(e, "blockify");
-        }
+        const int rc = launch_prep(p, ws, 0, p->total_ts, s);
+        if (rc != LAPH_OK) return rc;
         const laph::TcConfig cfg = tc_config(p);
         for (size_t ci = 0; ci < p->chunks.size(); ci++) {
             const int rc = launch_tc_chunk(p, ws, ci, cfg, s);
@@ -1512,7 +1499,7 @@ int laph_plan_launches_per_execute(const laph_plan *plan, int *n)
     if (!plan || !n) return LAPH_ERR_ARG;
     const int ptr_launches = (plan->n_inst + 63) / 64;
     if (is_tc_mode(plan->mode))
-        *n = ptr_launches + 2 * plan->n_inst /* scale, blockify */ +
+        *n = ptr_launches + 2 * ((plan->total_ts + 65534) / 65535) /* scale, blockify */ +
              3 * (int)plan->chunks.size() /* psi, contraction, FP64 site reduction */ +
              (!plan->chunks.empty() && plan->chunks.back().n_split > 0 &&
               plan->chunks.back().n_split < plan->chunks.back().n_units) /* a reduction for either kind of unit */;
@@ -1658,7 +1645,7 @@ static int execute_host_body(laph_plan *plan, const void *const *phi_host, void 
     for (size_t ci = 0; ci < nc; ci++) {
         const laph_plan::Chunk &c = plan->chunks[ci];
         CK(cudaStreamWaitEvent(s, plan->ev_in[ci], 0));
-        int rc = launch_chunk_prep(plan, ws, ci, s);
+        int rc = launch_prep(plan, ws, c.unit0, c.n_units, s);
         if (rc == LAPH_OK) rc = launch_tc_chunk(plan, ws, ci, cfg, s);
         if (rc != LAPH_OK) return rc;
         // the outputs of chunk ci are final once its site reduction (side stream) is done

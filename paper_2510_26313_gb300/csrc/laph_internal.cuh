@@ -166,24 +166,19 @@ __host__ __device__ inline int scale_exp(unsigned maxbits)
     int s = 126 - E;
     return s > 100 ? 100 : (s < -100 ? -100 : s);
 }
-// Max |field entry| per timeslice over all of an instance's fields (h_nfields[n] of them).
-cudaError_t launch_scale_max(const InstDev *d_inst, int n_inst, const int *h_ts_base, const int *h_T,
-                             const long long *h_elems, unsigned *d_maxbits, cudaStream_t s,
-                             const int *h_nfields = nullptr);
+// Max |field entry| of every unit's timeslice over all of its instance's fields
+// (n_fields, max_elems: the most of any unit).
+cudaError_t launch_scale_max(const InstDev *d_inst, const PsiUnit *d_units, int n_units, int n_fields,
+                             long long max_elems, unsigned *d_maxbits, cudaStream_t s);
 cudaError_t launch_diquarks(const float2 *phi, int L, int T, int N, float2 *out, cudaStream_t s);
 // Seeded pseudo-random complex entries in [-1, 1) (inputs the library makes itself).
 cudaError_t launch_fill_pattern(float2 *out, long long n, unsigned seed, cudaStream_t s);
 // acc[0] += sum |a - b|^2, acc[1] += sum |b|^2 (FP64; acc zeroed by the caller).
 cudaError_t launch_diff_norms(const void *a, bool a_c64, const double2 *b, long long n, double *acc, cudaStream_t s);
 cudaError_t launch_dense_fill(const double2 *packed, int T, int N, int P, double2 *dense, cudaStream_t s);
-// Site-blocked copies of phi_u (and, for triplets, phi_v).
-cudaError_t launch_blockify(const InstDev *d_inst, int inst, const InstDev &h, const unsigned *d_maxbits,
-                            cudaStream_t s);
-// The same for the timeslices [t0, t0 + nt) of one instance.
-cudaError_t launch_scale_max_range(const InstDev *d_inst, int inst, int t0, int nt, long long elems_per_ts,
-                                   unsigned *d_maxbits, cudaStream_t s, int n_fields = 1);
-cudaError_t launch_blockify_range(const InstDev *d_inst, int inst, const InstDev &h, int t0, int nt,
-                                  const unsigned *d_maxbits, cudaStream_t s);
+// Site-blocked copies of phi_u (and, for triplets, phi_v) of every unit (max_nblk: the most site blocks of any).
+cudaError_t launch_blockify(const InstDev *d_inst, const PsiUnit *d_units, int n_units, int max_nblk, bool triplets,
+                            const unsigned *d_maxbits, cudaStream_t s);
 
 // laph_simt.cu
 struct SimtConfig {

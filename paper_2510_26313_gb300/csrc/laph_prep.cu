@@ -175,14 +175,20 @@ cudaError_t launch_diff_norms(const void *a, bool a_c64, const double2 *b, long 
 // Largest |re|, |im| of phi per timeslice, as FP32 bits (non-negative floats
 // order like their bit patterns).  The tensor-core kernel turns it into an
 // exact power-of-two rescale before splitting into hi/lo halves.
-__global__ void scale_max_kernel(const InstDev *__restrict__ d_inst, int inst, int t0, unsigned *__restrict__ maxbits)
+//
+// One launch covers every (instance, timeslice) of the units given (and every
+// field): block (x, u, field) of unit u, grid-strided in x.  A ragged batch of
+// 24 instances took a launch of a few microseconds for each of them before.
+__global__ void __launch_bounds__(256) scale_max_kernel(const InstDev *__restrict__ d_inst,
+                                                        const PsiUnit *__restrict__ units, unsigned *__restrict__ maxbits)
 {
-    const InstDev &I = d_inst[inst];
-    const int t = t0 + blockIdx.y;
+    const PsiUnit un = units[blockIdx.y];
+    const InstDev &I = d_inst[un.inst];
+    if ((int)blockIdx.z >= I.n_fields) return;
     // field blockIdx.z: the column field (Nc vectors), then the row fields (N) of a multi-field instance
     const long long n = (long long)(blockIdx.z == 0 ? I.Nc : I.N) * I.V * 3;
     const float2 *f = blockIdx.z == 0 ? I.phi : (blockIdx.z == 1 ? I.phi_u : I.phi_v);
-    const float2 *base = f + (long long)t * n;
+    const float2 *base = f + (long long)un.t * n;
     float m = 0.f;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         float2 v = __ldg(base + e);
@@ -195,35 +201,24 @@ __global__ void scale_max_kernel(const InstDev *__restrict__ d_inst, int inst, i
     if (threadIdx.x < 32) {
         m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) atomicMax(maxbits + I.ts_base + t, __float_as_uint(m));
+        if (threadIdx.x == 0) atomicMax(maxbits + I.ts_base + un.t, __float_as_uint(m));
     }
 }
 
-cudaError_t launch_scale_max(const InstDev *d_inst, int n_inst, const int *h_ts_base, const int *h_T,
-                             const long long *h_elems, unsigned *d_maxbits, cudaStream_t s, const int *h_nfields)
+cudaError_t launch_scale_max(const InstDev *d_inst, const PsiUnit *d_units, int n_units, int n_fields,
+                             long long max_elems, unsigned *d_maxbits, cudaStream_t s)
 {
-    (void)h_ts_base;
-    for (int n = 0; n < n_inst; n++) {
-        long long blocks = (h_elems[n] + 256 * 8 - 1) / (256 * 8);
-        if (blocks > 256) blocks = 256;
-        if (blocks < 1) blocks = 1;
-        dim3 g((unsigned)blocks, (unsigned)h_T[n], (unsigned)(h_nfields ? h_nfields[n] : 1));
-        scale_max_kernel<<<g, 256, 0, s>>>(d_inst, n, 0, d_maxbits);
-        cudaError_t e = cudaGetLastError();
+    long long blocks = (max_elems + 256 * 8 - 1) / (256 * 8);
+    if (blocks > 256) blocks = 256;
+    if (blocks < 1) blocks = 1;
+    for (int u = 0; u < n_units; u += 65535) {
+        const int n = n_units - u < 65535 ? n_units - u : 65535;
+        scale_max_kernel<<<dim3((unsigned)blocks, (unsigned)n, (unsigned)n_fields), 256, 0, s>>>(d_inst, d_units + u,
+                                                                                                   d_maxbits);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-cudaError_t launch_scale_max_range(const InstDev *d_inst, int inst, int t0, int nt, long long elems_per_ts,
-                                   unsigned *d_maxbits, cudaStream_t s, int n_fields)
-{
-    long long blocks = (elems_per_ts + 256 * 8 - 1) / (256 * 8);
-    if (blocks > 256) blocks = 256;
-    if (blocks < 1) blocks = 1;
-    dim3 g((unsigned)blocks, (unsigned)nt, (unsigned)n_fields);
-    scale_max_kernel<<<g, 256, 0, s>>>(d_inst, inst, t0, d_maxbits);
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- site blocks
@@ -231,19 +226,37 @@ cudaError_t launch_scale_max_range(const InstDev *d_inst, int inst, int t0, int 
 // blk[t][b][n][e] = 2^s_t f[t][n][8b + e/3][e%3] for e < 24 (zero past V),
 // e = 24, 25 padding, with (f, blk) = (phi_u, phi_blk) for blockIdx.z = 0 and
 // (phi_v, blk_v) for blockIdx.z = 1 (triplets).  Memory bound: one read of
-// the field, one write of the copy.  Block (b, t) writes the N slots of site
-// block b (contiguous) and reads the 24 complex entries of each vector for
-// those sites (contiguous too).
-__global__ void __launch_bounds__(256) blockify_kernel(const InstDev *__restrict__ d_inst, int inst, int t0,
+// the field, one write of the copy.  Block (b, u) writes the N slots of site
+// block b of unit u (contiguous) and reads the 24 complex entries of each
+// vector for those sites (contiguous too): 16 bytes at a time where the field
+// is 16-byte aligned and V even (13 stores per slot instead of 26), else 8.
+// One launch covers all the units; blocks past an instance's own site
+// blocks return.
+__global__ void __launch_bounds__(256) blockify_kernel(const InstDev *__restrict__ d_inst,
+                                                       const PsiUnit *__restrict__ units,
                                                        const unsigned *__restrict__ maxbits)
 {
-    const InstDev &I = d_inst[inst];
-    const int b = blockIdx.x, t = t0 + blockIdx.y, N = I.N;
+    const PsiUnit un = units[blockIdx.y];
+    const InstDev &I = d_inst[un.inst];
+    const int b = blockIdx.x, t = un.t, N = I.N;
+    if (b >= I.nblk || (blockIdx.z && I.kind != INST_TRIPLETS)) return;
     const long long V = I.V;
     const float sc = __int_as_float((127 + scale_exp(maxbits[I.ts_base + t])) << 23);
     const float2 *src = (blockIdx.z ? I.phi_v : I.phi_u) + (long long)t * N * V * 3 + (long long)TC_BS * b * 3;
     float2 *dst = (blockIdx.z ? I.blk_v : I.phi_blk) + ((long long)t * I.nblk + b) * N * TC_SLOT;
     const int nvalid = (int)(V - (long long)TC_BS * b < TC_BS ? V - (long long)TC_BS * b : TC_BS) * 3;
+    if (!(V & 1) && !((uintptr_t)src & 15)) {
+        for (int idx = threadIdx.x; idx < N * (TC_SLOT / 2); idx += blockDim.x) {
+            const int n = idx / (TC_SLOT / 2), e = 2 * (idx - n * (TC_SLOT / 2));
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (e < nvalid) {   // nvalid is even with V
+                const float4 f = __ldg(reinterpret_cast<const float4 *>(src + (long long)n * V * 3 + e));
+                v = make_float4(f.x * sc, f.y * sc, f.z * sc, f.w * sc);
+            }
+            reinterpret_cast<float4 *>(dst)[idx] = v;
+        }
+        return;
+    }
     for (int idx = threadIdx.x; idx < N * TC_SLOT; idx += blockDim.x) {
         const int n = idx / TC_SLOT, e = idx - n * TC_SLOT;
         float2 v = make_float2(0.f, 0.f);
@@ -255,19 +268,14 @@ __global__ void __launch_bounds__(256) blockify_kernel(const InstDev *__restrict
     }
 }
 
-cudaError_t launch_blockify(const InstDev *d_inst, int inst, const InstDev &h, const unsigned *d_maxbits, cudaStream_t s)
+cudaError_t launch_blockify(const InstDev *d_inst, const PsiUnit *d_units, int n_units, int max_nblk, bool triplets,
+                            const unsigned *d_maxbits, cudaStream_t s)
 {
-    return launch_blockify_range(d_inst, inst, h, 0, h.T, d_maxbits, s);
-}
-
-cudaError_t launch_blockify_range(const InstDev *d_inst, int inst, const InstDev &h, int t0, int nt,
-                                  const unsigned *d_maxbits, cudaStream_t s)
-{
-    for (int tb = 0; tb < nt; tb += 65535) {
-        const int n = nt - tb < 65535 ? nt - tb : 65535;
-        dim3 g((unsigned)h.nblk, (unsigned)n, h.kind == INST_TRIPLETS ? 2u : 1u);
-        blockify_kernel<<<g, 256, 0, s>>>(d_inst, inst, t0 + tb, d_maxbits);
-        cudaError_t e = cudaGetLastError();
+    for (int u = 0; u < n_units; u += 65535) {
+        const int n = n_units - u < 65535 ? n_units - u : 65535;
+        blockify_kernel<<<dim3((unsigned)max_nblk, (unsigned)n, triplets ? 2u : 1u), 256, 0, s>>>(d_inst, d_units + u,
+                                                                                                 d_maxbits);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
