@@ -226,7 +226,8 @@ typedef struct {
     uint32_t seed;    /* start vectors (0: a fixed default) */
     int ts_group;     /* timeslices whose filter steps run back to back, so that their links and vectors stay
                          in L2 across the steps (0: as many as fill about 70% of the L2); d > 0 only */
-    int pdl;          /* 1: filter steps launched as programmatic dependents of their predecessors */
+    int pdl;          /* no effect: filter steps are always launched as programmatic dependents of their
+                         predecessors (1 used to ask for it) */
     int link_rows;    /* 2: read SU(3) links as their first two rows, the third rebuilt (used only if every
                          link is SU(3) to FP32 accuracy); 3: all three rows; 0: two rows unless the filter
                          groups fit in L2 */

@@ -252,8 +252,14 @@ __global__ void links_soa_kernel(const float2 *__restrict__ U, float2 *__restric
 // lap_kernel in the solver's layouts: out = a (-Delta in) + b in + c z.
 // Launched as a programmatic dependent of the previous step (a filter step
 // reads its predecessors' outputs and overwrites the vector read two steps
-// back): it lets the next grid be scheduled at once and waits for the full
-// completion of the previous grid before its first access to vectors.
+// back): a block lets the next grid be scheduled when its own arithmetic is
+// done, and reads its first links, which no step writes, before it waits for
+// the full completion of the previous grid, ahead of its first access to
+// vectors.  So the launch and one load latency of a step lie under the tail of
+// the step before.  (Scheduling the next grid from a block's first
+// instruction made its blocks take slots from the running grid: 48.0 ms of
+// filter steps at L=32, T=8, m=128, degree 48, against 44.3 without programmatic
+// launches and 43.9 this way; one timeslice 22.8, 16.1 and 14.7 ms.)
 // R12: the links are SU(3) and only their first two rows are read.  PAIRS:
 // the paired layouts above.
 template <bool R12, bool PAIRS>
@@ -263,8 +269,6 @@ __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(
                                                               int L, long long ts_in, long long ts_z, long long ts_out,
                                                               float a, float b, float c)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     // offsets within a timeslice are 32-bit (L <= 512: 9 V < 2^31); two
     // 32-bit divisions give the coordinates
     const unsigned uL = (unsigned)L, V = uL * uL * uL;
@@ -276,7 +280,10 @@ __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(
     const unsigned q1 = x / uL, c0 = x - q1 * uL, c2 = q1 / uL, c1 = q1 - c2 * uL;
     const unsigned cc[3] = {c0, c1, c2};
     const unsigned stride[3] = {1u, uL, uL * uL};
-    float2 fx[3], acc[3];
+    float2 fx[3], acc[3], uf[9], ub[9];
+    load_link<PAIRS, R12 ? 6 : 9>(Ut, V, x, uf);
+    load_link<PAIRS, R12 ? 6 : 9>(Ut, V, c0 == 0 ? x + (uL - 1) : x - 1, ub);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     load_site<PAIRS>(f, V, x, fx);
 #pragma unroll
     for (int q = 0; q < 3; q++) acc[q] = make_float2(0.f, 0.f);
@@ -286,11 +293,13 @@ __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(
         const unsigned dn = cc[mu] == 0 ? x + (uL - 1) * stride[mu] : x - stride[mu];
         const float2 *um = Ut + (long long)mu * 9 * V;
         // all loads of this direction issued before its multiply-adds
-        float2 fu[3], fd[3], uf[9], ub[9];
+        float2 fu[3], fd[3];
         load_site<PAIRS>(f, V, up, fu);
         load_site<PAIRS>(f, V, dn, fd);
-        load_link<PAIRS, R12 ? 6 : 9>(um, V, x, uf);
-        load_link<PAIRS, R12 ? 6 : 9>(um, V, dn, ub);
+        if (mu > 0) {
+            load_link<PAIRS, R12 ? 6 : 9>(um, V, x, uf);
+            load_link<PAIRS, R12 ? 6 : 9>(um, V, dn, ub);
+        }
         if (R12) {
             su3_third_row(uf);
             su3_third_row(ub);
@@ -306,6 +315,7 @@ __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(
     float2 *o = out + t * ts_out + (long long)n * V * 3;
     float2 zv[3] = {};
     if (z) load_site<PAIRS>(z + t * ts_z + (long long)n * V * 3, V, x, zv);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float2 r[3];
 #pragma unroll
     for (int q = 0; q < 3; q++) {
@@ -335,13 +345,17 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
 // registers; per row the products are summed in FP32 within the thread and
 // the warp (shuffles), the warps' partials in FP64 and across blocks with
 // FP64 atomics.  GB300's FP64 rate is a small fraction of its FP32 rate, so no
-// FP64 arithmetic runs per element.
+// FP64 arithmetic runs per element.  Block z takes its share of the rows
+// (rows_z, a multiple of DOT_JC): the sums of different rows do not meet, and a
+// few timeslices alone are little more than one wave of blocks (T=8 at L=32:
+// 384 on 304 places).
 constexpr int DOT_EPT = 8;      // elements of w per thread
 constexpr int DOT_JC = 32;      // rows between flushes of the warp partials
 constexpr int DOT_RG = 4;       // rows whose loads are issued together
 __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restrict__ basis, long long ts_basis,
                                                            const float2 *__restrict__ w, long long ts_w, long long K,
-                                                           int nj, double2 *__restrict__ dots, int dots_stride)
+                                                           int nj, int rows_z, double2 *__restrict__ dots,
+                                                           int dots_stride)
 {
     __shared__ float2 part[LAP_THREADS / 32][DOT_JC];
     const int t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -353,8 +367,9 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
         const long long e = e0 + (long long)q * LAP_THREADS;
         wv[q] = e < K ? w[t * ts_w + e] : make_float2(0.f, 0.f);
     }
-    for (int j0 = 0; j0 < nj; j0 += DOT_JC) {
-        const int jn = min(DOT_JC, nj - j0);
+    const int j_end = min(nj, ((int)blockIdx.z + 1) * rows_z);
+    for (int j0 = blockIdx.z * rows_z; j0 < j_end; j0 += DOT_JC) {
+        const int jn = min(DOT_JC, j_end - j0);
         for (int jj = 0; jj < jn; jj += DOT_RG) {
             float2 b[DOT_RG][DOT_EPT];
 #pragma unroll
@@ -398,10 +413,14 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
 // Gram-Schmidt update, w[t] -= sum_j coef[t][j] basis[t][j] for j < nj, with
 // the coefficients rounded to FP32 in shared memory (dynamic, nj float2) and
 // FP32 multiply-adds; UPD_EPT elements per thread, the loads of UPD_RG rows
-// issued together.  norm (may be null): norm[t] += |w[t]|^2 of the result.
+// issued together.  norm (may be null): norm[t] += |w[t]|^2 of the result.  Two
+// rows at a time at six blocks per SM keep as much in flight as four at four,
+// and fill the chip more evenly when there are few timeslices (T=8 at L=32: 768
+// blocks on 608 places before).  With the split rows of dots_kernel the
+// orthogonalisation of T=8, m=128 went from 39.8 to 36.5 ms.
 constexpr int UPD_EPT = 4;
-constexpr int UPD_RG = 4;
-__global__ void __launch_bounds__(LAP_THREADS) update_kernel(const float2 *__restrict__ basis, long long ts_basis,
+constexpr int UPD_RG = 2;
+__global__ void __launch_bounds__(LAP_THREADS, 6) update_kernel(const float2 *__restrict__ basis, long long ts_basis,
                                                              float2 *__restrict__ w, long long ts_w, long long K, int nj,
                                                              const double2 *__restrict__ coef, int coef_stride,
                                                              double *__restrict__ norm)
@@ -859,7 +878,6 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
     const bool group_in_l2 = d > 0 && (double)tg * 8 * 42 * V <= 0.7 * l2;
     st.ts_group = d > 0 ? tg : T;
     const bool want_r12 = prm->link_rows == 2 || (prm->link_rows == 0 && !group_in_l2);
-    const bool pdl = prm->pdl != 0;
     bool r12 = false;
     // paired layouts where every block they split into is 16-byte aligned
     const bool pairs = V % 2 == 0;
@@ -915,14 +933,14 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
                 auto at = [&](const float2 *base, long long ts) { return base + (long long)t0 * ts; };
                 float2 *y1 = d == 1 ? w : ya;
                 e = launch_lap_soa(Ug, at(v, ts_v), nullptr, (float2 *)at(y1, K), L, nt, 1, ts_v, 0, K,
-                                     (float)(1.0 / cheb_e), (float)(-cheb_c / cheb_e), 0.f, cs, r12, pairs, pdl && t0 > 0);
+                                     (float)(1.0 / cheb_e), (float)(-cheb_c / cheb_e), 0.f, cs, r12, pairs, t0 > 0);
                 const float2 *prev = v;
                 long long ts_prev = ts_v;
                 float2 *cur = y1;
                 for (int k = 2; k <= d && e == cudaSuccess; k++) {
                     float2 *dst = k == d ? w : (cur != ya && prev != ya ? ya : (cur != yb && prev != yb ? yb : yc));
                     e = launch_lap_soa(Ug, at(cur, K), at(prev, ts_prev), (float2 *)at(dst, K), L, nt, 1, K, ts_prev,
-                                         K, (float)(2.0 / cheb_e), (float)(-2.0 * cheb_c / cheb_e), -1.f, cs, r12, pairs, pdl);
+                                         K, (float)(2.0 / cheb_e), (float)(-2.0 * cheb_c / cheb_e), -1.f, cs, r12, pairs, true);
                     prev = cur;
                     ts_prev = K;
                     cur = dst;
@@ -944,6 +962,15 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
             if (filter) return cudaGraphLaunch(filter, s);
             return filter_launches(s);
         };
+        // inner products of w with basis vectors [0, nj), the rows shared out until there are a few waves of blocks
+        auto launch_dots = [&](int nj) {
+            const long long want = 6LL * 152, have = (long long)blocks_dot * T;
+            const int chunks = (nj + DOT_JC - 1) / DOT_JC;
+            const int nz = (int)std::max(1LL, std::min<long long>(chunks, (want + have - 1) / have));
+            const int rows_z = (chunks + nz - 1) / nz * DOT_JC;
+            dots_kernel<<<dim3(blocks_dot, T, (nj + rows_z - 1) / rows_z), LAP_THREADS, 0, s>>>(basis, ts_b, w, K, K, nj,
+                                                                                               rows_z, dots, m + 1);
+        };
         // removes from w its components along basis vectors [0, nj), twice
         // ("twice is enough"); the first pass's coefficients land in h_dots,
         // |w|^2 of the result in h_norm.  Synchronises the stream.
@@ -953,7 +980,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
                 e = cudaMemsetAsync(dots, 0, sizeof(double2) * (m + 1) * T, s);
                 if (e == cudaSuccess && pass == 1) e = cudaMemsetAsync(dnorm, 0, sizeof(double) * T, s);
                 if (e != cudaSuccess) break;
-                dots_kernel<<<dim3(blocks_dot, T), LAP_THREADS, 0, s>>>(basis, ts_b, w, K, K, nj, dots, m + 1);
+                launch_dots(nj);
                 update_kernel<<<dim3(blocks_upd, T), LAP_THREADS, sizeof(float2) * nj, s>>>(
                     basis, ts_b, w, K, K, nj, dots, m + 1, pass == 1 ? dnorm : nullptr);
                 e = cudaGetLastError();
@@ -969,7 +996,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
         auto norm_w = [&]() -> cudaError_t {
             cudaError_t e = cudaMemsetAsync(dots, 0, sizeof(double2) * T, s);
             if (e == cudaSuccess) {
-                dots_kernel<<<dim3(blocks_dot, T), LAP_THREADS, 0, s>>>(w, K, w, K, K, 1, dots, 1);
+                dots_kernel<<<dim3(blocks_dot, T), LAP_THREADS, 0, s>>>(w, K, w, K, K, 1, DOT_JC, dots, 1);
                 e = cudaGetLastError();
                 st.launches++;
             }
@@ -990,7 +1017,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
                 e = cudaMemsetAsync(dots, 0, sizeof(double2) * (m + 1) * T, s);
                 if (e == cudaSuccess && pass == 1) e = cudaMemsetAsync(dnorm, 0, sizeof(double) * T, s);
                 if (e != cudaSuccess) break;
-                dots_kernel<<<dim3(blocks_dot, T), LAP_THREADS, 0, s>>>(basis, ts_b, w, K, K, j + 1, dots, m + 1);
+                launch_dots(j + 1);
                 update_kernel<<<dim3(blocks_upd, T), LAP_THREADS, sizeof(float2) * (j + 1), s>>>(
                     basis, ts_b, w, K, K, j + 1, dots, m + 1, pass == 1 ? dnorm : nullptr);
                 if (pass == 0) take_alpha_kernel<<<bt, 128, 0, s>>>(dots, m + 1, j, dalpha, m, T);
