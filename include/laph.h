@@ -309,9 +309,9 @@ typedef struct {
                         to a multiple of 8): a tile covers one block, its running sums become one FP32 partial per
                         output, and the partials of all blocks are added in FP64 in block order */
     int tile_cols;   /* tensor-core modes: complex columns per tile: 104, 96, 80 or 64 in layout 0; 176 (default),
-                        192, 208 or 128 in layout 1.  0 with layout 0: the plan takes the shape (either layout) with the
-                        lowest estimated time, 104 or 96 columns of layout 0 for small problems; every shape gives
-                        the same results */
+                        192, 208 or 128 in layout 1.  0 with layout 0: the plan takes the shape (either layout, or tiles
+                        of 128 rows x 208 columns worked by pairs of CTAs) with the lowest estimated time, 104 or 96
+                        columns of layout 0 for small problems; every shape gives the same results */
     int layout;      /* tensor-core modes: how the complex product is laid out on the real tensor cores.
                         0: every complex column of the phased operand is two real rows (re, im) of the
                         MMA's B operand, 128 complex rows per tile; 1: every complex row of the diquark / meson
@@ -425,7 +425,7 @@ LAPH_API int laph_plan_tensor_flops(const laph_plan *plan, double *flops);
 /* One candidate schedule timed by LAPH_PLAN_AUTOTUNE. */
 typedef struct {
     int tile_cols;                  /* complex columns per tile */
-    int layout;                     /* laph_plan_options.layout */
+    int layout;                     /* laph_plan_options.layout, or 2: pairs of CTAs (128 rows x 208 columns a pair) */
     int sum_sites;                  /* sites per block of the FP64 site reduction */
     int chunk_sites;                /* drain interval of the tensor core's FP32 accumulation, in sites */
     int chunk_sites_b;              /* drain interval of the tiles without meson rows, in sites */
@@ -441,7 +441,7 @@ typedef struct {
  * (pseudo-random entries in [-1, 1); inputs, outputs and a workspace are
  * allocated for the duration; one warm-up and one timed execute each) by a
  * coordinate search: tile shape (layout 0 with 104, 96, 80 and 64 columns, layout 1
- * with 176, 192, 208 and 128 columns) x tile order x chunking
+ * with 176, 192, 208 and 128 columns, CTA pairs) x tile order x chunking
  * (the wave model and, for one instance, the largest chunk within the 24 GiB
  * cap); then, from the fastest, half and twice the site-block size of the
  * FP64 reduction; then half and 1.5 times the drain interval (for all

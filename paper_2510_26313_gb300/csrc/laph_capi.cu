@@ -82,6 +82,7 @@ constexpr size_t SPLIT_MAX_BYTES = 1ull << 30;
 // layout 1, 208 / 176 / 128 columns: 0.747 / 0.698 / 0.636) and to the B-operand
 // pass (bytes written and read per us).
 constexpr double STAGE_US = 0.45, STAGE_US_COL = 0.00137;
+constexpr double PAIR_STAGE_US = 0.46, PAIR_STAGE_US_COL = 0.00137;   // CTA pairs: 0.746 us at 208 columns
 constexpr double RING_COST = 1.11;
 constexpr double PSI_BYTES_US = 6.3e6, PSI_BYTES_US_ROWS2 = 5.3e6;
 constexpr double SHAPE_MARGIN = 0.03;
@@ -100,7 +101,7 @@ struct Sched {
     int tile_cols, sum_sites, chunk_sites;
     long long per_chunk;
     int order;
-    int rows2;           // 1: the row-doubled layout of the complex product (64 complex rows per tile)
+    int rows2;           // 1: the row-doubled layout of the complex product (64 complex rows per tile); 2: CTA pairs
     int chunk_sites_b;   // drain interval of tiles without meson rows (0: chunk_sites)
 };
 }  // namespace laph
@@ -431,7 +432,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     auto build_tiles = [&](int TC, int rows2) {
         p->tile_cols = TC;
         p->rows2 = tc ? rows2 : 0;
-        p->tile_rows = !tc ? laph::SIMT_TR : (rows2 ? laph::TC_TR_ROWS2 : laph::TC_TR);
+        p->tile_rows = !tc ? laph::SIMT_TR : (rows2 == 1 ? laph::TC_TR_ROWS2 : laph::TC_TR);
         const int TR = p->tile_rows;
         const int skip_step = rows2 ? 16 : 8;   // column skips keep the UMMA N a multiple of 16
         p->max_staged = 0;
@@ -512,6 +513,8 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     };
     int sms = 0;
     PCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    // persistent workers that claim tiles: CTAs, or pairs of CTAs
+    auto workers = [&]() { return std::max(1, p->rows2 == 2 ? sms / 2 : sms); };
     // units per chunk: one instance -> the count (within the cap) that
     // leaves the fewest partly filled waves of persistent CTAs (want_largest:
     // the largest count within the cap); several instances -> chunks filled
@@ -529,7 +532,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             long long best = -1, best_rounds = 0;
             for (long long n = 1; n <= n_max; n++) {
                 const long long full = U / n, rest = U % n;
-                const long long rounds = full * ((n * tpu + sms - 1) / sms) + (rest * tpu + sms - 1) / sms;
+                const long long w = workers(), rounds = full * ((n * tpu + w - 1) / w) + (rest * tpu + w - 1) / w;
                 if (best < 0 || rounds <= best_rounds) {
                     best = n;
                     best_rounds = rounds;
@@ -657,7 +660,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             const int terms = (mode == LAPH_MODE_TC_F16X3 || mode == LAPH_MODE_TC_BF16X3) ? 3 : 1;
             for (const TileDev &u : tiles) {
                 const int n_real = p->rows2 ? ((u.ncols + 15) & ~15) - u.cskip : 2 * ((u.ncols + 7) & ~7) - 2 * u.cskip;
-                p->mma_flops += 2.0 * laph::TC_TR * n_real * (2 * laph::TC_KSTAGE) * terms * u.nst;
+                p->mma_flops += 2.0 * laph::TC_TR * (p->rows2 == 2 ? 2 : 1) * n_real * (2 * laph::TC_KSTAGE) * terms * u.nst;
             }
         }
         p->h_units = units;
@@ -674,7 +677,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     auto last_chunk_time = [&](int n_split, size_t *extra_bytes) -> double {
         const int cs = drain_stages();
         const laph_plan::Chunk &c = p->chunks.back();
-        std::vector<long long> free_at(sms, 0);   // a heap, earliest first
+        std::vector<long long> free_at(workers(), 0);   // a heap, earliest first
         const auto later = std::greater<long long>();
         long long end = 0, total = 0, longest = 0;
         *extra_bytes = 0;
@@ -698,7 +701,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
                 }
             }
         }
-        if (n_split) end = std::max(end, total / sms + longest);
+        if (n_split) end = std::max(end, total / workers() + longest);
         return (double)end + 2.0 * (double)*extra_bytes / SPLIT_BYTES_PER_STAGE;
     };
     // The tables of a schedule, with as many trailing units of the last chunk
@@ -720,7 +723,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
         }
         const laph_plan::Chunk last = p->chunks.back();
         int best = 0;
-        if ((p->chunk_sites_b == 0 || p->chunk_sites_b == p->chunk_sites) && last.n_tiles <= (long long)SPLIT_MAX_WAVES * sms) {
+        if ((p->chunk_sites_b == 0 || p->chunk_sites_b == p->chunk_sites) && last.n_tiles <= (long long)SPLIT_MAX_WAVES * workers()) {
             size_t extra = 0;
             double best_t = last_chunk_time(0, &extra) * (1.0 - SPLIT_MARGIN);
             for (int u = 1; u <= last.n_units; u = u < 4 || u == last.n_units ? u + 1 : std::min(2 * u, last.n_units)) {
@@ -814,7 +817,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
         long long n_tiles = 0;
         auto stage_us = [&](const TileDev &u) {
             const int n_real = r2 ? ((u.ncols + 15) & ~15) - u.cskip : 2 * ((u.ncols + 7) & ~7) - 2 * u.cskip;
-            return STAGE_US + STAGE_US_COL * n_real;
+            return r2 == 2 ? PAIR_STAGE_US + PAIR_STAGE_US_COL * n_real : STAGE_US + STAGE_US_COL * n_real;
         };
         for (int n = 0; n < n_inst; n++) {
             const InstDev &d = p->h_inst[n];
@@ -822,9 +825,9 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             n_tiles += (long long)ones[n].size() * d.n_sc * d.T;
             bytes += (double)d.T * ((double)d.n_ct * d.n_st * laph::tc_stage_bytes(nc, r2) + 24.0 * d.Nc * d.V);
         }
-        double us = total / sms;
-        if (n_tiles <= (long long)SPLIT_MAX_WAVES * sms) {
-            std::vector<double> free_at(sms, 0.0);
+        double us = total / workers();
+        if (n_tiles <= (long long)SPLIT_MAX_WAVES * workers()) {
+            std::vector<double> free_at(workers(), 0.0);
             const auto later = std::greater<double>();
             double end = 0.0;
             for (int n = 0; n < n_inst; n++) {
@@ -838,7 +841,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
                             std::push_heap(free_at.begin(), free_at.end(), later);
                         }
             }
-            us = std::min(end, n_tiles >= 2 * sms ? 1.04 * us : (1.0 + TILE_STAGES / 16.0) * us);
+            us = std::min(end, n_tiles >= 2 * workers() ? 1.04 * us : (1.0 + TILE_STAGES / 16.0) * us);
         }
         return us * (ring < 4 ? RING_COST : 1.0) + bytes / (r2 ? PSI_BYTES_US_ROWS2 : PSI_BYTES_US);
     };
@@ -847,7 +850,8 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     // with enough work takes another shape where the estimate is better by
     // SHAPE_MARGIN: layout 1 has half the B-operand bytes and 64-row tiles
     // (meson rows alone fill half of a 128-row tile), a narrower tile of layout 0
-    // may cover the columns in as many tiles.  Every shape gives the same bits.
+    // may cover the columns in as many tiles, CTA pairs keep a stage ring of four
+    // buffers with many row vectors.  Every shape gives the same bits.
     if (tc && !opt_cols && !opt_layout) {
         const double us104 = shape_us(def.tile_cols, 0);
         if (laph::tc_ring_depth(p->max_staged, def.tile_cols, 0) < 4 &&
@@ -858,7 +862,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             stages += (long long)ones[n].size() * p->h_inst[n].n_st * p->h_inst[n].T;
         if (stages >= (long long)SHAPE_MIN_STAGES * sms) {
             double best = (def.tile_cols == 96 ? shape_us(96, 0) : us104) * (1.0 - SHAPE_MARGIN);
-            const std::pair<int, int> shapes[] = {{96, 0}, {80, 0}, {64, 0}, {208, 1}, {176, 1}, {128, 1}};
+            const std::pair<int, int> shapes[] = {{96, 0}, {80, 0}, {64, 0}, {208, 1}, {176, 1}, {128, 1}, {laph::TC_PAIR_COLS, 2}};
             for (const auto &sh : shapes) {
                 const double us = shape_us(sh.first, sh.second);
                 if (us < best) {
@@ -975,7 +979,7 @@ static int merge_drains(laph_plan *plan)
             }
             const int n_real =
                 plan->rows2 ? ((v.ncols + 15) & ~15) - v.cskip : 2 * ((v.ncols + 7) & ~7) - 2 * v.cskip;
-            flops += 2.0 * laph::TC_TR * n_real * (2 * laph::TC_KSTAGE) * terms * v.nst;
+            flops += 2.0 * laph::TC_TR * (plan->rows2 == 2 ? 2 : 1) * n_real * (2 * laph::TC_KSTAGE) * terms * v.nst;
             tiles.push_back(v);
         }
         c.tile0 = tile0;
@@ -1315,7 +1319,7 @@ static int autotune(laph_plan *p, const laph::Sched &def, const std::function<cu
         // 1: tile width x tile order x chunking (the largest chunk only for one instance)
         const bool one_inst = p->n_inst == 1 && !(p->flags & LAPH_PLAN_CHUNK_PER_TIMESLICE);
         const std::pair<int, int> shapes[] = {{def.tile_cols, def.rows2}, {104, 0}, {96, 0},  {80, 0}, {64, 0},
-                                              {176, 1},           {192, 1}, {208, 1}, {128, 1}};
+                                              {176, 1},           {192, 1}, {208, 1}, {128, 1}, {laph::TC_PAIR_COLS, 2}};
         for (size_t k = 0; k < sizeof(shapes) / sizeof(shapes[0]); k++) {
             const int nc = shapes[k].first, r2 = shapes[k].second;
             if (k > 0 && nc == def.tile_cols && r2 == def.rows2) continue;

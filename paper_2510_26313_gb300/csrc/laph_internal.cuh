@@ -193,7 +193,7 @@ cudaError_t launch_simt(const InstDev *d_inst, const TileDev *d_tiles, long long
 struct TcConfig {
     int elem;          // 0 = FP16 hi/lo, 1 = BF16 hi/lo
     int ncols;         // tile width in complex columns: 104, 96, 80 or 64; row-doubled layout 208, 192, 176 or 128
-    int rows2;         // 1: row-doubled layout (two real A rows per complex row, 64 complex rows per tile)
+    int rows2;         // 1: row-doubled layout (two real A rows per complex row, 64 complex rows per tile); 2: CTA pairs
     int terms;         // 3 (split) or 1 (plain)
     int chunk_sites;   // sites accumulated by the tensor core between FP32 drains
     int chunk_sites_b; // the same for tiles without meson rows
@@ -208,6 +208,7 @@ constexpr int TC_KSTAGE = 3 * TC_BS;  // complex K entries per stage: one site b
 // (nc in the row-doubled layout) x 48 FP16 each.
 constexpr int tc_stage_bytes(int nc, bool rows2 = false) { return 2 * (rows2 ? nc : 2 * nc) * (2 * TC_KSTAGE) * 2; }
 constexpr int TC_TR_ROWS2 = 64;   // complex rows per tile in the row-doubled layout
+constexpr int TC_PAIR_COLS = 208;  // complex columns per tile of CTA pairs (128 complex rows; rows2 = 2)
 // Tile widths with compiled kernels for each layout.
 bool tc_shape_supported(int ncols, int rows2);
 constexpr int TC_MAX_STAGED = 160;  // staged row vectors per tile

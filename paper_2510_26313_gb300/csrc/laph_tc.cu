@@ -61,6 +61,8 @@
 // there.
 // Every wait on an mbarrier is bounded; on expiry the CTA records
 // STATUS_TIMEOUT, raises a shared abort flag and all roles return.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -413,7 +415,8 @@ __device__ __forceinline__ int next_tile(const Ctx c, Ring &rt, bool &ok)
 // column-doubled layout; in the row-doubled layout 1 (re, -im) for the re-row
 // and 2 (im, re) for the im-row of a complex row, so that with B rows
 // (Psi_re, Psi_im) the re-row gives the real part of the product and the
-// im-row its imaginary part.
+// im-row its imaginary part.  3 (im, -re): the im-row against B rows
+// (Psi_re, -Psi_im) (CTA pairs, whose re-rows have form 0).
 template <int ELEM, int FORM>
 __device__ __forceinline__ void a_quarter(int kind, const uint8_t *pu, const uint8_t *pv, uint32_t (&hi)[12],
                                           uint32_t (&lo)[12])
@@ -442,6 +445,7 @@ __device__ __forceinline__ void a_quarter(int kind, const uint8_t *pu, const uin
                 d = make_float2(0.f, 0.f);
             if (FORM == 1) d = make_float2(d.x, -d.y);
             if (FORM == 2) d = make_float2(d.y, d.x);
+            if (FORM == 3) d = make_float2(d.y, -d.x);
             split2<ELEM>(d.x, d.y, hi[6 * m + e], lo[6 * m + e]);
         }
     }
@@ -875,6 +879,473 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
     }
 }
 
+// ------------------------------------------------------------ CTA pairs
+
+// The same contraction by pairs of CTAs (clusters of two, cta_group::2): a tile
+// is 128 complex rows x PAIR_NC complex columns of one site block, and one MMA
+// (M = 256) works for both SMs.  CTA 0 holds the re-rows of the tile's complex
+// rows, CTA 1 their im-rows, each 128 real A rows in its own tensor memory; the
+// B operand has one real row (Psi_re, -Psi_im) per complex column, and each CTA
+// stages every other group of eight columns, so that a pair has the tile area of
+// two 128 x 104 tiles with half of the B bytes, in shared memory, in L2 and in
+// the B-operand pass, and half of the MMA's shared-memory reads.  Against the
+// re-rows' A = (a_re, a_im) the im-rows' is (a_im, -a_re).
+//
+// Roles as in tc_kernel (column-doubled warp counts).  CTA 0's loader claims
+// the pair's tiles and hands them to both CTAs; its MMA warp issues for both,
+// and its commits arrive on the barriers of both (multicast).  The producers'
+// and epilogue warps' arrivals for the MMA warp, and every reader's for the
+// tile ring, go to CTA 0.  The accumulator is drained whole: all its columns
+// are committed together, and the next chunk starts when both CTAs have
+// drained them.
+//
+// The half-size B stage leaves a ring of four buffers where tc_kernel's is
+// three deep (more than about 80 row vectors per tile), which is what it is
+// used for: L=48, N=128, 33 momenta, one timeslice: contraction 68.2 -> 66.0 ms,
+// B-operand pass 3.65 -> 2.60 ms.  With four buffers on both sides the two run
+// alike (three fields, L=32, N=64: 7.73 against 7.75 ms): the period of a stage
+// is set by the producers and the power limit, not by the B operand.
+constexpr int PAIR_NC = TC_PAIR_COLS;
+constexpr int PAIR_HALF_BYTES = PAIR_NC * (2 * TC_KSTAGE) * 2;      // one CTA's half of a stage image, hi + lo
+constexpr int PAIR_B_BYTES = PAIR_HALF_BYTES / 2;                   // hi (or lo) of it
+constexpr int PAIR_ATOM_BYTES = PAIR_B_BYTES / KSTEPS;              // one k-step
+constexpr int PAIR_READERS = (N_AWARPS + 8 + 1) + (N_AWARPS + 8 + 2);
+static_assert(PAIR_NC % 16 == 0 && 2 * PAIR_NC <= (int)A_COL, "tile width within the tensor-memory budget");
+static_assert(2 * PAIR_HALF_BYTES == tc_stage_bytes(PAIR_NC, true), "stage image size");
+
+__device__ __forceinline__ uint32_t cta_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Cluster address of the same shared-memory object in CTA `rank`.
+__device__ __forceinline__ uint32_t peer_addr(const void *p, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+
+// Arrival on a barrier of either CTA.  The plain form orders what these
+// arrivals order: tensor-memory accesses (with the tcgen05 fences) and the use
+// of a ring slot.  Cluster-scope release and acquire, which wait for memory
+// traffic, are kept for the tile ring's entries, once per tile.
+__device__ __forceinline__ void mbar_arrive_at(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// warp_wait with acquire at cluster scope: for barriers that the other CTA's
+// threads arrive on.
+__device__ __forceinline__ bool warp_wait_cluster(const Ctx c, uint64_t *bar, uint32_t parity)
+{
+    if (!__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) {
+        if (!warp_wait_slow(c.S, c.status, c.lane, bar, parity)) return false;
+        mbar_try_wait_cluster(bar, parity);   // the phase is complete: acquires at cluster scope
+    }
+    return true;
+}
+
+__device__ __forceinline__ int next_tile_pair(const Ctx c, Ring &rt, bool &ok)
+{
+    if (!warp_wait_cluster(c, &c.S->tfull[rt.slot], rt.phase)) {
+        ok = false;
+        return -1;
+    }
+    const int t = *(volatile int *)&c.S->tile_ring[rt.slot];
+    __syncwarp();
+    if (c.lane == 0) mbar_arrive_at(peer_addr(&c.S->tempty[rt.slot], 0));
+    rt.next(TRING);
+    return t;
+}
+
+// M = 256 over the pair: 128 rows in each CTA.
+__device__ __forceinline__ uint32_t idesc_pair(int n_real, int bf16)
+{
+    return (1u << 4) | ((uint32_t)bf16 << 7) | ((uint32_t)bf16 << 10) | ((uint32_t)(n_real >> 3) << 17) |
+           ((uint32_t)(256 >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_pair(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrives on the barrier at this offset in both CTAs.
+__device__ __forceinline__ void commit_pair(uint64_t *bar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
+template <int ELEM, int TERMS>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREADS, 1) tc_pair_kernel(const KParams kp)
+{
+    using R = Roles<false>;
+    constexpr int WARP_LOAD = R::WARP_LOAD, WARP_MMA = R::WARP_MMA;
+    constexpr uint32_t SUM_COL = PAIR_NC;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int NS = kp.ns;
+    Shared *S = reinterpret_cast<Shared *>(smem + NS * kp.stage_bytes);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cta_rank();
+    const Ctx c{S, kp.status, lane};
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < NS; s++) {
+            mbar_init(&S->full[s], 1);
+            mbar_init(&S->full[NS + s], 1);
+            mbar_init(&S->empty[s], 1);
+        }
+        for (int s = 0; s < TRING; s++) {
+            mbar_init(&S->tfull[s], 1);
+            mbar_init(&S->tempty[s], PAIR_READERS);
+        }
+        for (int s = 0; s < 2; s++) mbar_init(&S->a_full[s], 2 * N_AGROUP);
+        mbar_init(&S->acc_full[0], 1);
+        mbar_init(&S->acc_empty[0], 2 * R::EPI_WARPS);
+        mbar_init(&S->done, 1);
+        S->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == WARP_MMA) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S->tmem_base)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        tc_fence_before();
+    }
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem = S->tmem_base;
+
+    if (warp == WARP_LOAD) {
+        // ---------------------------------------------------------- loader
+        Ring rs{0, 0}, rf{0, 0}, rt{0, 0};   // stage buffer, data barrier, tile ring
+        uint32_t n_issued = 0;   // stages whose copies were issued
+        bool ok = true;
+        while (ok) {
+            int tile = 0;
+            if (rank == 0) {
+                if (!warp_wait(c, &S->tempty[rt.slot], rt.phase ^ 1u)) break;
+                if (lane == 0) {
+                    tile = (int)atomicAdd(kp.counter, 1u);
+                    if (tile >= kp.n_tiles) tile = -1;
+                    *(volatile int *)&S->tile_ring[rt.slot] = tile;
+                    mbar_arrive(&S->tfull[rt.slot]);
+                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(&S->tile_ring[rt.slot], 1)), "r"(tile)
+                                 : "memory");
+                    mbar_arrive_release_cluster(peer_addr(&S->tfull[rt.slot], 1));
+                }
+                tile = __shfl_sync(0xffffffffu, tile, 0);
+                rt.next(TRING);
+            } else {
+                tile = next_tile_pair(c, rt, ok);
+            }
+            if (tile < 0) break;
+            const TileDev td = kp.tiles[tile];
+            const InstDev &I = kp.insts[td.inst];
+            const int nst = td.nst;
+            const uint32_t bytesA = td.nv * SLOT_BYTES, bytesW = td.nw * SLOT_BYTES;
+            const uint8_t *bsrc = kp.psi + td.psi_off + (long long)td.s0 * (2 * PAIR_HALF_BYTES) + rank * PAIR_HALF_BYTES;
+            const long long blk0 = ((long long)td.t * I.nblk + td.s0) * I.N;
+            const float2 *asrc = I.phi_blk + (blk0 + td.v_lo) * TC_SLOT;
+            const float2 *wsrc = I.blk_v + (blk0 + td.w_lo) * TC_SLOT;
+            const long long astep = (long long)I.N * TC_SLOT;
+            for (int st = 0; st < nst; st++) {
+                if (!warp_wait(c, &S->empty[rs.slot], rs.phase ^ 1u)) {
+                    ok = false;
+                    break;
+                }
+                if (lane == 0) {
+                    uint8_t *buf = smem + rs.slot * kp.stage_bytes;
+                    uint64_t *fb = &S->full[rf.slot];
+                    mbar_arrive_expect_tx(fb, PAIR_HALF_BYTES + bytesA + bytesW);
+                    bulk_g2s(buf, bsrc + (long long)st * (2 * PAIR_HALF_BYTES), PAIR_HALF_BYTES, fb);
+                    bulk_g2s(buf + PAIR_HALF_BYTES, asrc + st * astep, bytesA, fb);
+                    if (bytesW) bulk_g2s(buf + PAIR_HALF_BYTES + bytesA, wsrc + st * astep, bytesW, fb);
+                }
+                __syncwarp();
+                rs.next(NS);
+                rf.next(2 * NS);
+                n_issued++;
+            }
+        }
+        for (uint32_t k = n_issued > (uint32_t)NS ? n_issued - NS : 0; k < n_issued; k++)
+            drain_wait(S, kp.status, lane, &S->full[k % (2 * NS)], (k / (2 * NS)) & 1u);
+    } else if (warp < N_AWARPS) {
+        // ---------------------------------------------------------- A producers
+        const int quad = warp & 3, half = (warp >> 2) & 1, grp = warp >> 3;
+        const int r = quad * 32 + lane;
+        const uint32_t ta0 = tmem + ((uint32_t)(quad * 32) << 16) + A_COL + (uint32_t)grp * A_SLOT_COLS + 12u * half;
+        const uint32_t a_full0 = peer_addr(&S->a_full[grp], 0);
+        uint32_t G = 0;   // global index of the tile's first stage
+        bool stalled = false, ok = true;
+        Ring rt{0, 0};
+        while (ok) {
+            const int tile = next_tile_pair(c, rt, ok);
+            if (tile < 0) break;
+            const TileDev td = kp.tiles[tile];
+            const InstDev &I = kp.insts[td.inst];
+            const int nst = td.nst;
+            const int gr = td.row0 + r;
+            int kind = 0, vi = 0, vj = 0;
+            const bool trip = I.kind == INST_TRIPLETS;
+            if (gr < I.mes_rows) {
+                kind = 1;
+                vi = gr;
+            } else if (gr < I.rows) {
+                kind = 2;
+                const int q = gr - I.mes_rows;
+                if (trip) {
+                    vi = q / I.N;
+                    vj = q - vi * I.N;
+                } else {
+                    pair_of(q, vi, vj);
+                }
+            }
+            const int si = kind ? vi - td.v_lo : 0;
+            const int sj = kind == 2 ? (trip ? td.nv + vj - td.w_lo : vj - td.v_lo) : 0;
+            const int off_u = PAIR_HALF_BYTES + si * SLOT_BYTES + half * HALF_BYTES;
+            const int off_v = PAIR_HALF_BYTES + sj * SLOT_BYTES + half * HALF_BYTES;
+            int st = (grp - (int)(G & 1u)) & 1;
+            const uint32_t Gs = G + st;
+            int s = (int)(Gs % (uint32_t)NS);
+            int sf = (int)(Gs % (uint32_t)(2 * NS));
+            uint32_t ph = (Gs / (uint32_t)(2 * NS)) & 1u;
+            const uint32_t Gp = Gs + (uint32_t)NS - 2u;
+            int s2 = (int)(Gp % (uint32_t)NS);
+            uint32_t ph2 = ((Gp / (uint32_t)NS) & 1u) ^ 1u;
+            for (; st < nst; st += 2) {
+                if (!warp_wait(c, &S->full[sf], ph)) {
+                    ok = false;
+                    break;
+                }
+                const uint8_t *buf = smem + s * kp.stage_bytes;
+                uint32_t hi[12], lo[12];
+                if (rank == 0)
+                    a_quarter<ELEM, 0>(kind, buf + off_u, buf + off_v, hi, lo);
+                else
+                    a_quarter<ELEM, 3>(kind, buf + off_u, buf + off_v, hi, lo);
+                if (!warp_wait(c, &S->empty[s2], ph2)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                a_store(ta0, hi, lo);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                const bool skip = kp.debug_stall && !stalled && blockIdx.x == 0 && warp == 0;
+                if (skip) stalled = true;
+                if (lane == 0 && !skip) mbar_arrive_at(a_full0);
+                s += 2;
+                if (s >= NS) s -= NS;
+                sf += 2;
+                if (sf >= 2 * NS) {
+                    sf -= 2 * NS;
+                    ph ^= 1u;
+                }
+                s2 += 2;
+                if (s2 >= NS) {
+                    s2 -= NS;
+                    ph2 ^= 1u;
+                }
+            }
+            G += (uint32_t)nst;
+        }
+    } else if (warp < WARP_LOAD) {
+        // ---------------------------------------------------------- epilogue
+        const int quad = warp & 3, eh = (warp - N_AWARPS) >> 2;
+        const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+        const uint32_t empty0 = peer_addr(&S->acc_empty[0], 0);
+        uint32_t g = 0;   // drains done
+        bool ok = true;
+        Ring rt{0, 0};
+        while (ok) {
+            const int tile = next_tile_pair(c, rt, ok);
+            if (tile < 0) break;
+            const TileDev td = kp.tiles[tile];
+            const InstDev &I = kp.insts[td.inst];
+            const int n_real = acc_cols<true>(td.ncols, td.cskip);
+            const int cs = td.row0 >= I.mes_rows ? kp.chunk_stages_b : kp.chunk_stages;
+            const int n_ch = (td.nst + cs - 1) / cs;
+            for (int ch = 0; ch < n_ch; ch++) {
+                if (!warp_wait(c, &S->acc_full[0], g & 1u)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                for (int b = eh; b * 16 < n_real; b += 2) {
+                    uint32_t va[16], vs[16];
+                    tmem_ld16(tmem + lane_base + ACC_COL + 16u * b, va);
+                    if (ch > 0) tmem_ld16(tmem + lane_base + SUM_COL + 16u * b, vs);
+                    tmem_wait_ld();
+                    if (ch > 0) {
+#pragma unroll
+                        for (int e = 0; e < 16; e++)
+                            va[e] = __float_as_uint(__uint_as_float(va[e]) + __uint_as_float(vs[e]));
+                    }
+                    tmem_st16(tmem + lane_base + SUM_COL + 16u * b, va);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_at(empty0);
+                g++;
+            }
+            if (!ok) break;
+            // tile done (see tc_kernel): this CTA's part, real or imaginary, of
+            // the tile's rows.  Accumulator columns [0, n_real / 2) are the even
+            // groups of eight tile columns, the others the odd ones.
+            const long long N = I.N;
+            const int P = I.P, gr = td.row0 + quad * 32 + lane;
+            const bool rvalid = gr < I.rows, meson = gr < I.mes_rows, trip = I.kind == INST_TRIPLETS;
+            const int q = gr - I.mes_rows;
+            int pi_ = 0, pj = 0;
+            if (rvalid && !meson && !trip) pair_of(q, pi_, pj);
+            const bool tri = !meson && !trip;
+            const long long step = meson ? N * I.Nc : (trip ? N * N * N : I.n_trip);
+            const long long row_off = meson ? I.n_outB + (long long)gr * I.Nc : (trip ? q * N : q);
+            const int k_min = !rvalid ? 0x7fffffff : (tri ? pj + 1 : 0);
+            float *part = reinterpret_cast<float *>(kp.part + td.part_off + row_off) + rank;
+            const int n_grp = n_real / 16;
+            for (int b = eh; b * 16 < n_real; b += 2) {
+                uint32_t v[16];
+                tmem_ld16(tmem + lane_base + SUM_COL + 16u * b, v);
+                tmem_wait_ld();
+#pragma unroll 1
+                for (int h = 0; h < 2; h++) {
+                    const int grp8 = 2 * b + h, odd = grp8 >= n_grp;
+                    const int cc0 = td.cskip + 8 * (2 * (grp8 - odd * n_grp) + odd);
+                    int k = (td.col0 + cc0) / P, p = td.col0 + cc0 - k * P;
+                    long long e = p * step + (tri ? binom3(k) : k);
+#pragma unroll 1
+                    for (int u = 0; u < 8; u++) {
+                        if (cc0 + u < td.ncols && k >= k_min) part[2 * e] = __uint_as_float(v[8 * h + u]);
+                        e += step;
+                        if (++p == P) {
+                            p = 0;
+                            e += (tri ? binom2(k) : 1) - P * step;
+                            k++;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    } else if (rank == 0) {
+        // ---------------------------------------------------------- MMA issue
+        Ring rs{0, 0}, ra{0, 0};
+        uint32_t g = 0;   // chunks
+        bool ok = true;
+        Ring rt{0, 0};
+        while (ok) {
+            const int tile = next_tile_pair(c, rt, ok);
+            if (tile < 0) break;
+            const TileDev td = kp.tiles[tile];
+            const int nst = td.nst;
+            const int chunk = td.row0 >= kp.insts[td.inst].mes_rows ? kp.chunk_stages_b : kp.chunk_stages;
+            const uint32_t idesc = idesc_pair(acc_cols<true>(td.ncols, td.cskip), ELEM);
+            // cskip / 2 of each CTA's B rows are not needed: 32 bytes each per k-step
+            const uint64_t bskip = (uint64_t)(td.cskip * 16) >> 4;
+            int cs = 0;   // stage within the current accumulation chunk
+            for (int st = 0; st < nst; st++) {
+                const bool chunk_end = cs + 1 == chunk || st + 1 == nst;
+                if (cs == 0 && !warp_wait(c, &S->acc_empty[0], (g & 1u) ^ 1u)) {
+                    ok = false;
+                    break;
+                }
+                if (!warp_wait(c, &S->a_full[ra.slot], ra.phase)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                if (lane == 0) {
+                    const uint32_t a_hi = tmem + A_COL + (uint32_t)ra.slot * A_SLOT_COLS, a_lo = a_hi + A_LO;
+                    const uint64_t dhi = desc_sw32(smem_u32(smem + rs.slot * kp.stage_bytes)) + bskip;
+                    const uint64_t dlo = dhi + (uint64_t)(PAIR_B_BYTES >> 4);
+#pragma unroll
+                    for (int ks = 0; ks < KSTEPS; ks++) {
+                        const uint64_t koff = (uint64_t)ks * (PAIR_ATOM_BYTES >> 4);
+                        mma_pair(tmem + ACC_COL, a_hi + 8 * ks, dhi + koff, idesc, ks == 0 ? (cs != 0) : 1u);
+                        if (TERMS == 3) {
+                            mma_pair(tmem + ACC_COL, a_hi + 8 * ks, dlo + koff, idesc, 1u);
+                            mma_pair(tmem + ACC_COL, a_lo + 8 * ks, dhi + koff, idesc, 1u);
+                        }
+                    }
+                    if (chunk_end) commit_pair(&S->acc_full[0]);
+                    commit_pair(&S->empty[rs.slot]);   // the stage buffers and A slots of both CTAs
+                }
+                __syncwarp();
+                if (chunk_end) {
+                    g++;
+                    cs = 0;
+                } else {
+                    cs++;
+                }
+                rs.next(NS);
+                ra.next(2);
+            }
+        }
+        // every issued MMA has completed before tensor memory is released
+        if (lane == 0) commit_pair(&S->done);
+        __syncwarp();
+        warp_wait(c, &S->done, 0u);
+    } else {
+        // CTA 1's idle MMA warp follows the tiles, so that its wait for the last
+        // commit is a short one
+        Ring rt{0, 0};
+        bool ok = true;
+        while (ok && next_tile_pair(c, rt, ok) >= 0) {
+        }
+        warp_wait(c, &S->done, 0u);
+    }
+
+    __syncthreads();
+    cluster_sync_all();   // neither CTA leaves or frees tensor memory while the other may reach into it
+    if (warp == WARP_MMA) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+}
+
 // ------------------------------------------------------------ B stage images
 
 // Job = (unit, column tile ct, `group` consecutive stages; TC_PSI_GROUP, fewer where a launch has few jobs); the
@@ -888,14 +1359,15 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
 // image, in the K-major 32-byte-swizzled layout the contraction's
 // descriptors expect.  Every store instruction of a warp writes sixteen
 // whole 32-byte rows.
-template <int ELEM, int NC, bool RD>
+template <int ELEM, int NC, bool RD, bool PAIR>
 __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__ insts, const PsiUnit *__restrict__ units,
                                                      int n_units, long long n_jobs, int group,
                                                      const unsigned *__restrict__ maxbits,
                                                      uint8_t *__restrict__ psi)
 {
     using SH = Shape<NC, RD>;
-    constexpr int BIMG_BYTES = SH::BIMG_BYTES, B_BYTES = SH::B_BYTES, ATOM_COL_BYTES = SH::ATOM_COL_BYTES;
+    constexpr int BIMG_BYTES = SH::BIMG_BYTES, B_BYTES = PAIR ? PAIR_B_BYTES : SH::B_BYTES;
+    constexpr int ATOM_COL_BYTES = PAIR ? PAIR_ATOM_BYTES : SH::ATOM_COL_BYTES;
     const int cu = threadIdx.x >> 1, j = threadIdx.x & 1;
     for (long long job = blockIdx.x; job < n_jobs; job += gridDim.x) {
         int lo = 0, hi = n_units - 1;
@@ -927,8 +1399,9 @@ __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__
         const float2 *phk = I.phi + ((long long)un.t * I.Nc + k) * V * 3;
         uint8_t *img = psi + un.psi_off + ((long long)ct * n_st + st0) * BIMG_BYTES;
         // real B rows of the column: re-row 2 cu and im-row 2 cu + 1, or (row-doubled layout) row cu
-        const int n0 = RD ? cu : 2 * cu, n1 = n0 + 1;
-        const uint32_t o0 = sw32(n0, j), o1 = sw32(n1, j);
+        // (CTA pairs: row 8 (a / 2) + cu % 8 of the half a % 2, a = cu / 8 the group of eight columns)
+        const int n0 = PAIR ? (cu >> 4) * 8 + (cu & 7) : (RD ? cu : 2 * cu), n1 = n0 + 1;
+        const uint32_t o0 = sw32(n0, j) + (PAIR ? ((cu >> 3) & 1) * PAIR_HALF_BYTES : 0), o1 = sw32(n1, j);
         for (int st = st0; st < st1; st++, img += BIMG_BYTES) {
 #pragma unroll
             for (int ks = 0; ks < KSTEPS; ks++) {
@@ -950,8 +1423,8 @@ __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__
                     uint32_t h, l;
                     split2<ELEM>(z.x, z.y, h, l);
                     if (RD) {
-                        rh[v] = h;                          // (re, im)
-                        rl[v] = l;
+                        rh[v] = PAIR ? h ^ 0x80000000u : h;   // (re, im), CTA pairs (re, -im)
+                        rl[v] = PAIR ? l ^ 0x80000000u : l;
                     } else {
                         rh[v] = h ^ 0x80000000u;            // (re, -im)
                         rl[v] = l ^ 0x80000000u;
@@ -1180,20 +1653,51 @@ cudaError_t launch_one(const InstDev *d_inst, const TileDev *d_tiles, long long 
     return cudaGetLastError();
 }
 
-template <int NC, bool RD>
+// Stage ring of the pair kernel: a CTA's half of the image and the row vectors.
+int pair_stage_bytes(int max_staged) { return (PAIR_HALF_BYTES + max_staged * SLOT_BYTES + 1023) & ~1023; }
+
+int pair_ring_depth(int max_staged)
+{
+    for (int ns = MAX_NS; ns >= 2; ns--)
+        if (smem_for(ns, pair_stage_bytes(max_staged)) <= SMEM_LIMIT) return ns;
+    return 0;
+}
+
+template <int ELEM, int TERMS>
+cudaError_t launch_pair(const InstDev *d_inst, const TileDev *d_tiles, long long n_tiles, const unsigned *maxbits,
+                        const uint8_t *psi, float2 *part, unsigned *counter, const TcConfig &cfg, int *status,
+                        cudaStream_t s)
+{
+    KParams kp = {d_inst, d_tiles, maxbits, psi, part, counter, status, (int)n_tiles, 0, 0, 0, 0, cfg.debug_stall};
+    kp.chunk_stages = std::max(1, cfg.chunk_sites * 3 / KSTAGE);
+    kp.chunk_stages_b = std::max(1, (cfg.chunk_sites_b > 0 ? cfg.chunk_sites_b : cfg.chunk_sites) * 3 / KSTAGE);
+    kp.stage_bytes = pair_stage_bytes(cfg.max_staged);
+    kp.ns = pair_ring_depth(cfg.max_staged);
+    if (!kp.ns) return cudaErrorNotSupported;
+    const int smem = smem_for(kp.ns, kp.stage_bytes);
+    const cudaError_t e =
+        cudaFuncSetAttribute(tc_pair_kernel<ELEM, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const long long pairs = std::min<long long>(std::max(1, cfg.grid / 2), n_tiles);
+    tc_pair_kernel<ELEM, TERMS><<<(unsigned)(2 * pairs), Roles<false>::NTHREADS, smem, s>>>(kp);
+    return cudaGetLastError();
+}
+
+template <int NC, bool RD, bool PAIR = false>
 void psi_launch(int elem, unsigned grid, const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs,
                 int group, const unsigned *d_maxbits, uint8_t *psi, cudaStream_t s)
 {
     if (elem == 0)
-        psi_kernel<0, NC, RD><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
+        psi_kernel<0, NC, RD, PAIR><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
     else
-        psi_kernel<1, NC, RD><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
+        psi_kernel<1, NC, RD, PAIR><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
 }
 
 }  // namespace
 
 int tc_ring_depth(int max_staged, int ncols, int rows2)
 {
+    if (rows2 == 2) return pair_ring_depth(max_staged);
     const int sb = stage_bytes_for(max_staged, ncols, rows2 != 0);
     for (int ns = MAX_NS; ns >= 2; ns--)
         if (smem_for(ns, sb) <= SMEM_LIMIT) return ns;
@@ -1222,6 +1726,16 @@ cudaError_t launch_tc(const InstDev *d_inst, const TileDev *d_tiles, long long n
             return launch_one<0, 1, NC, RD>(d_inst, d_tiles, n_tiles, d_maxbits, psi, part, counter, cfg, d_status, s); \
         if (cfg.elem == 1 && cfg.terms == 1)                                                                    \
             return launch_one<1, 1, NC, RD>(d_inst, d_tiles, n_tiles, d_maxbits, psi, part, counter, cfg, d_status, s); \
+    }
+    if (cfg.rows2 == 2 && cfg.ncols == PAIR_NC) {
+#define LAPH_PAIR_CASE(E, TM)                                                                                  \
+    if (cfg.elem == E && cfg.terms == TM)                                                                      \
+        return launch_pair<E, TM>(d_inst, d_tiles, n_tiles, d_maxbits, psi, part, counter, cfg, d_status, s);
+        LAPH_PAIR_CASE(0, 3)
+        LAPH_PAIR_CASE(1, 3)
+        LAPH_PAIR_CASE(0, 1)
+        LAPH_PAIR_CASE(1, 1)
+#undef LAPH_PAIR_CASE
     }
     LAPH_TC_CASE(104, false)
     LAPH_TC_CASE(96, false)
@@ -1264,13 +1778,15 @@ cudaError_t launch_psi(const InstDev *d_inst, const PsiUnit *d_units, int n_unit
         psi_launch<80, false>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else if (!rows2 && ncols == 64)
         psi_launch<64, false>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
-    else if (rows2 && ncols == 208)
+    else if (rows2 == 2 && ncols == PAIR_NC)
+        psi_launch<PAIR_NC, true, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
+    else if (rows2 == 1 && ncols == 208)
         psi_launch<208, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
-    else if (rows2 && ncols == 192)
+    else if (rows2 == 1 && ncols == 192)
         psi_launch<192, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
-    else if (rows2 && ncols == 176)
+    else if (rows2 == 1 && ncols == 176)
         psi_launch<176, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
-    else if (rows2 && ncols == 128)
+    else if (rows2 == 1 && ncols == 128)
         psi_launch<128, true>(elem, grid, d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi, s);
     else
         return cudaErrorNotSupported;
