@@ -1359,8 +1359,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
 // image, in the K-major 32-byte-swizzled layout the contraction's
 // descriptors expect.  Every store instruction of a warp writes sixteen
 // whole 32-byte rows.
+//
+// Bound by the stage images' writes in layout 0; with one row per column
+// (row-doubled layout, CTA pairs) a load feeds half as many stores, and the
+// load latency of three k-steps one after the other showed.  So all of a
+// stage's loads are issued before its arithmetic, 16 bytes at a time where the
+// field is aligned, and a block takes half of such a job's columns, so that
+// about 1000 threads fit an SM (416 a block left two blocks of them).  L=32, 19
+// momenta: 64 vectors x 16 timeslices at 208 columns 3.44 -> 2.89 ms (4.8 ->
+// 5.7 TB/s), 10 timeslices 2.21 -> 1.88 ms; projection 1.07 -> 1.00 ms; L=48, 33
+// momenta, 128 vectors 2.64 -> 2.35 ms; layout 0 at 104 columns 0.342 -> 0.328 ms.
+
+// Columns of a job that one block takes: half of a job's where a column is one
+// B row (twice as many columns as in layout 0).
+constexpr int psi_cols(int nc, bool rd) { return rd ? nc / 2 : nc; }
+
 template <int ELEM, int NC, bool RD, bool PAIR>
-__global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__ insts, const PsiUnit *__restrict__ units,
+__global__ void __launch_bounds__(2 * psi_cols(NC, RD), 1200 / (2 * psi_cols(NC, RD))) psi_kernel(const InstDev *__restrict__ insts, const PsiUnit *__restrict__ units,
                                                      int n_units, long long n_jobs, int group,
                                                      const unsigned *__restrict__ maxbits,
                                                      uint8_t *__restrict__ psi)
@@ -1368,8 +1383,9 @@ __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__
     using SH = Shape<NC, RD>;
     constexpr int BIMG_BYTES = SH::BIMG_BYTES, B_BYTES = PAIR ? PAIR_B_BYTES : SH::B_BYTES;
     constexpr int ATOM_COL_BYTES = PAIR ? PAIR_ATOM_BYTES : SH::ATOM_COL_BYTES;
-    const int cu = threadIdx.x >> 1, j = threadIdx.x & 1;
-    for (long long job = blockIdx.x; job < n_jobs; job += gridDim.x) {
+    constexpr int SPLIT = NC / psi_cols(NC, RD);   // blocks per job; the grid is a multiple of it
+    const int cu = (threadIdx.x >> 1) + (int)(blockIdx.x % SPLIT) * psi_cols(NC, RD), j = threadIdx.x & 1;
+    for (long long job = blockIdx.x / SPLIT; job < n_jobs; job += gridDim.x / SPLIT) {
         int lo = 0, hi = n_units - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -1402,24 +1418,41 @@ __global__ void __launch_bounds__(2 * NC) psi_kernel(const InstDev *__restrict__
         // (CTA pairs: row 8 (a / 2) + cu % 8 of the half a % 2, a = cu / 8 the group of eight columns)
         const int n0 = PAIR ? (cu >> 4) * 8 + (cu & 7) : (RD ? cu : 2 * cu), n1 = n0 + 1;
         const uint32_t o0 = sw32(n0, j) + (PAIR ? ((cu >> 3) & 1) * PAIR_HALF_BYTES : 0), o1 = sw32(n1, j);
+        const bool vec = !(V & 1) && !((uintptr_t)I.phi & 15);   // every row of the field is 16-byte aligned
         for (int st = st0; st < st1; st++, img += BIMG_BYTES) {
+            // all loads of the stage before its arithmetic: k-step ks takes entries e0 .. e0+3 of the stage,
+            // sites 8 st + (e0 + v) / 3
+            float2 fs[KSTEPS][4], ws[KSTEPS][2];
 #pragma unroll
             for (int ks = 0; ks < KSTEPS; ks++) {
-                // entries e0 .. e0+3 of the stage: sites 8 st + (e0 + v) / 3
                 const int e0 = 8 * ks + 4 * j;
                 const int xs = 8 * st + e0 / 3, c0 = e0 % 3;
-                float2 f[4], w[2];
+                if (vec && valid && 8 * st + 8 <= V) {
+                    const float4 *pf = reinterpret_cast<const float4 *>(phk + 24 * (long long)st + e0);
+                    const float4 fa = __ldg(pf), fb = __ldg(pf + 1);
+                    fs[ks][0] = make_float2(fa.x, fa.y);
+                    fs[ks][1] = make_float2(fa.z, fa.w);
+                    fs[ks][2] = make_float2(fb.x, fb.y);
+                    fs[ks][3] = make_float2(fb.z, fb.w);
+                } else {
 #pragma unroll
-                for (int v = 0; v < 4; v++) {
-                    const int x = xs + (c0 + v) / 3;
-                    f[v] = (valid && x < V) ? __ldg(phk + 3 * x + (c0 + v) % 3) : make_float2(0.f, 0.f);
+                    for (int v = 0; v < 4; v++) {
+                        const int x = xs + (c0 + v) / 3;
+                        fs[ks][v] = (valid && x < V) ? __ldg(phk + 3 * x + (c0 + v) % 3) : make_float2(0.f, 0.f);
+                    }
                 }
 #pragma unroll
-                for (int q = 0; q < 2; q++) w[q] = (valid && xs + q < V) ? __ldg(ph + xs + q) : make_float2(0.f, 0.f);
+                for (int q = 0; q < 2; q++)
+                    ws[ks][q] = (valid && xs + q < V) ? __ldg(ph + xs + q) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int ks = 0; ks < KSTEPS; ks++) {
+                const int c0 = (8 * ks + 4 * j) % 3;
                 uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
                 for (int v = 0; v < 4; v++) {
-                    const float2 z = cmulf(w[(c0 + v) / 3], make_float2(f[v].x * sc, f[v].y * sc));
+                    const float2 f = fs[ks][v], w = c0 + v >= 3 ? ws[ks][1] : ws[ks][0];
+                    const float2 z = cmulf(w, make_float2(f.x * sc, f.y * sc));
                     uint32_t h, l;
                     split2<ELEM>(z.x, z.y, h, l);
                     if (RD) {
@@ -1687,10 +1720,12 @@ template <int NC, bool RD, bool PAIR = false>
 void psi_launch(int elem, unsigned grid, const InstDev *d_inst, const PsiUnit *d_units, int n_units, long long n_jobs,
                 int group, const unsigned *d_maxbits, uint8_t *psi, cudaStream_t s)
 {
+    constexpr int cols = psi_cols(NC, RD);
+    grid *= NC / cols;
     if (elem == 0)
-        psi_kernel<0, NC, RD, PAIR><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
+        psi_kernel<0, NC, RD, PAIR><<<grid, 2 * cols, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
     else
-        psi_kernel<1, NC, RD, PAIR><<<grid, 2 * NC, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
+        psi_kernel<1, NC, RD, PAIR><<<grid, 2 * cols, 0, s>>>(d_inst, d_units, n_units, n_jobs, group, d_maxbits, psi);
 }
 
 }  // namespace
