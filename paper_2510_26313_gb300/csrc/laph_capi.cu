@@ -1023,12 +1023,14 @@ static laph::TcConfig tc_config(const laph_plan *p)
     return cfg;
 }
 
-// The side stream and one pair of events per chunk (made outside any stream
+// The side stream (of a plan of several chunks) and one pair of events per chunk (made outside any stream
 // capture: at plan creation and before each autotuning candidate).
 static cudaError_t ensure_side(laph_plan *p)
 {
     cudaError_t e;
-    if (!p->side && (e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking)) != cudaSuccess) return e;
+    if (p->chunks.size() > 1 && !p->side &&
+        (e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking)) != cudaSuccess)
+        return e;
     while (p->ev_tc.size() < p->chunks.size()) {
         cudaEvent_t a = nullptr, b = nullptr;
         if ((e = cudaEventCreateWithFlags(&a, cudaEventDisableTiming)) != cudaSuccess) return e;
@@ -1045,12 +1047,12 @@ static cudaError_t ensure_side(laph_plan *p)
 // B-operand pass, contraction and FP64 site reduction of chunk ci (tensor-core
 // path), with the timing events of LAPH_PLAN_TIMING around each launch.  The
 // reduction runs on the plan's side stream after the contraction (event
-// ev_tc[ci]); the contraction of chunk ci waits for the reduction of chunk
-// ci - 1, which reads the same partial buffer (event ev_red[ci - 1]).  The
-// caller joins ev_red of the last chunk back into `s`.
+// ev_tc[ci]), the last chunk's on `s`; the contraction of chunk ci waits for
+// the reduction of chunk ci - 1, which reads the same partial buffer (event
+// ev_red[ci - 1]), so that everything is back in `s` at the end.
 static int launch_tc_chunk(laph_plan *p, char *ws, size_t ci, const laph::TcConfig &cfg, cudaStream_t s)
 {
-    if (!p->side || p->ev_tc.size() < p->chunks.size()) return LAPH_ERR_ARG;
+    if ((p->chunks.size() > 1 && !p->side) || p->ev_tc.size() < p->chunks.size()) return LAPH_ERR_ARG;
     cudaError_t e;
     const bool timing = !p->ev_begin.empty();
     unsigned *maxbits = (unsigned *)(ws + p->off_maxbits);
@@ -1077,14 +1079,18 @@ static int launch_tc_chunk(laph_plan *p, char *ws, size_t ci, const laph::TcConf
         CK(cudaEventRecord(p->ev_end[cs], s));
         p->n_timed++;
     }
-    CK(cudaEventRecord(p->ev_tc[ci], s));
-    CK(cudaStreamWaitEvent(p->side, p->ev_tc[ci], 0));
-    if (timing) CK(cudaEventRecord(p->rd_begin[cs], p->side));
+    // the last chunk has nothing left to run beside its reduction
+    const cudaStream_t rs = ci + 1 < p->chunks.size() ? p->side : s;
+    if (rs != s) {
+        CK(cudaEventRecord(p->ev_tc[ci], s));
+        CK(cudaStreamWaitEvent(rs, p->ev_tc[ci], 0));
+    }
+    if (timing) CK(cudaEventRecord(p->rd_begin[cs], rs));
     e = laph::launch_reduce(p->d_inst, p->d_units + c.unit0, c.n_units, c.n_split, c.n_red, c.n_red_split, maxbits, part,
-                            p->side);
+                            rs);
     if (e != cudaSuccess) return cuda_fail(e, "site reduction");
-    if (timing) CK(cudaEventRecord(p->rd_end[cs], p->side));
-    CK(cudaEventRecord(p->ev_red[ci], p->side));
+    if (timing) CK(cudaEventRecord(p->rd_end[cs], rs));
+    CK(cudaEventRecord(p->ev_red[ci], rs));
     return LAPH_OK;
 }
 
@@ -1106,14 +1112,15 @@ static int launch_prep(laph_plan *p, char *ws, int unit0, int n_units, cudaStrea
     return LAPH_OK;
 }
 
-static int launch_batch(laph_plan *p, void *workspace, cudaStream_t s)
+// cleared: the pointer upload has cleared the counters and scales already
+static int launch_batch(laph_plan *p, void *workspace, cudaStream_t s, bool cleared = false)
 {
     cudaError_t e;
     const bool timing = !p->ev_begin.empty();
     if (is_tc_mode(p->mode)) {
         if (!workspace || ((uintptr_t)workspace) % 256) return LAPH_ERR_WORKSPACE;
         char *ws = (char *)workspace;
-        CK(cudaMemsetAsync(ws, 0, p->ws_zero_bytes, s));
+        if (!cleared) CK(cudaMemsetAsync(ws, 0, p->ws_zero_bytes, s));
         const int rc = launch_prep(p, ws, 0, p->total_ts, s);
         if (rc != LAPH_OK) return rc;
         const laph::TcConfig cfg = tc_config(p);
@@ -1121,7 +1128,6 @@ static int launch_batch(laph_plan *p, void *workspace, cudaStream_t s)
             const int rc = launch_tc_chunk(p, ws, ci, cfg, s);
             if (rc != LAPH_OK) return rc;
         }
-        if (!p->chunks.empty()) CK(cudaStreamWaitEvent(s, p->ev_red[p->chunks.size() - 1], 0));
     } else {
         laph::SimtConfig cfg;
         cfg.chunk_sites = p->chunk_sites;
@@ -1527,10 +1533,13 @@ int laph_plan_execute(laph_plan *plan, const void *const *phi, void *const *out_
     CK(cudaGetDevice(&cur));
     if (cur != plan->device) return LAPH_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    const bool tc = is_tc_mode(plan->mode);
+    if (tc && (!workspace || ((uintptr_t)workspace) % 256)) return LAPH_ERR_WORKSPACE;
     cudaError_t e = laph::launch_set_pointers(plan->d_inst, 0, plan->n_inst, phi, needB ? out_B : nullptr,
-                                              needM ? out_M : nullptr, workspace, s);
+                                              needM ? out_M : nullptr, workspace, s, nullptr, 1, workspace,
+                                              tc ? plan->ws_zero_bytes : 0);
     if (e != cudaSuccess) return cuda_fail(e, "set_pointers");
-    return launch_batch(plan, workspace, s);
+    return launch_batch(plan, workspace, s, true);
 }
 
 int laph_plan_execute_fields(laph_plan *plan, const void *const *fields, void *const *out, void *workspace,
@@ -1548,10 +1557,12 @@ int laph_plan_execute_fields(laph_plan *plan, const void *const *fields, void *c
     CK(cudaGetDevice(&cur));
     if (cur != plan->device) return LAPH_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    if (!workspace || ((uintptr_t)workspace) % 256) return LAPH_ERR_WORKSPACE;
     cudaError_t e = laph::launch_set_pointers(plan->d_inst, 0, plan->n_inst, nullptr, trip ? out : nullptr,
-                                              trip ? nullptr : out, workspace, s, fields, nf);
+                                              trip ? nullptr : out, workspace, s, fields, nf, workspace,
+                                              plan->ws_zero_bytes);
     if (e != cudaSuccess) return cuda_fail(e, "set_pointers");
-    return launch_batch(plan, workspace, s);
+    return launch_batch(plan, workspace, s, true);
 }
 
 int laph_plan_host_workspace_size(const laph_plan *plan, size_t *bytes)
@@ -1668,7 +1679,6 @@ static int execute_host_body(laph_plan *plan, const void *const *phi_host, void 
             }
         }
     }
-    if (nc > 0) CK(cudaStreamWaitEvent(s, plan->ev_red[nc - 1], 0));
     CK(cudaStreamSynchronize(plan->d2h));
     CK(cudaStreamSynchronize(s));
     return LAPH_OK;

@@ -153,10 +153,12 @@ cudaError_t launch_phase_table(int L, const int32_t *d_mom, int P, double2 *out6
                                cudaStream_t s);
 // fields: null (every instance has one field, phi[n]), else n_fields entries
 // per instance in the order (phi, psi, chi) for triplets, (phi, psi) for
-// doublets; phi may then be null.
+// doublets; phi may then be null.  The launch also clears zero_bytes bytes at
+// `zero` (16-byte aligned, a multiple of 16).
 cudaError_t launch_set_pointers(InstDev *d_inst, int first, int count, const void *const *phi,
                                 void *const *outB, void *const *outM, void *workspace, cudaStream_t s,
-                                const void *const *fields = nullptr, int n_fields = 1);
+                                const void *const *fields = nullptr, int n_fields = 1, void *zero = nullptr,
+                                size_t zero_bytes = 0);
 // Power-of-two exponent s with max|phi| * 2^s in [0.5, 1), from the FP32 bits of max|phi|.
 __host__ __device__ inline int scale_exp(unsigned maxbits)
 {

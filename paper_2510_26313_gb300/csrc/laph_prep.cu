@@ -44,6 +44,8 @@ constexpr int PTR_BATCH = 64;
 struct PtrBatch {
     int first, count;
     char *ws;
+    unsigned *zero;   // words cleared by the launch (16-byte aligned, a multiple of 4)
+    int n_zero;
     const void *phi[PTR_BATCH];    // column field
     const void *phi_u[PTR_BATCH];  // first row field
     const void *phi_v[PTR_BATCH];  // second row field
@@ -54,6 +56,7 @@ struct PtrBatch {
 __global__ void set_pointers_kernel(InstDev *d_inst, PtrBatch b)
 {
     const int n = threadIdx.x;
+    for (int i = 4 * n; i < b.n_zero; i += 4 * PTR_BATCH) *reinterpret_cast<uint4 *>(b.zero + i) = make_uint4(0u, 0u, 0u, 0u);
     if (n < b.count) {
         InstDev &I = d_inst[b.first + n];
         I.phi = (const float2 *)b.phi[n];
@@ -68,11 +71,13 @@ __global__ void set_pointers_kernel(InstDev *d_inst, PtrBatch b)
 
 cudaError_t launch_set_pointers(InstDev *d_inst, int first, int count, const void *const *phi, void *const *outB,
                                 void *const *outM, void *workspace, cudaStream_t s, const void *const *fields,
-                                int n_fields)
+                                int n_fields, void *zero, size_t zero_bytes)
 {
     for (int base = 0; base < count; base += PTR_BATCH) {
         PtrBatch b;
         b.ws = (char *)workspace;
+        b.zero = (unsigned *)zero;
+        b.n_zero = base == 0 ? (int)(zero_bytes / sizeof(unsigned)) : 0;
         b.first = first + base;
         b.count = count - base < PTR_BATCH ? count - base : PTR_BATCH;
         for (int n = 0; n < b.count; n++) {
