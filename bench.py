@@ -132,7 +132,9 @@ def schedule_of(plan, tuned: bool) -> dict:
     """The tensor-core schedule a plan runs (and, when autotuned, every candidate it timed)."""
     d = plan.describe()
     sch = plan.schedule()
-    out = {"layout": 1 if d["tile_rows"] == 64 else 0, "tile_cols": d["tile_cols"], "tile_rows": d["tile_rows"],
+    # 0: column-doubled, 1: row-doubled, 2: pairs of CTAs (128 rows x 208 columns)
+    layout = 1 if d["tile_rows"] == 64 else 2 if d["tile_cols"] > 104 else 0
+    out = {"layout": layout, "tile_cols": d["tile_cols"], "tile_rows": d["tile_rows"],
            "chunk_sites": d["chunk_sites"], "chunk_sites_b": plan.drain_sites()[1], "sum_sites": plan.sum_sites()[0],
            "timeslices_per_chunk": sch["timeslices_per_chunk"], "tile_order": sch["tile_order"], "autotuned": tuned}
     if tuned:
@@ -992,7 +994,8 @@ def main():
         peak = float(peaks.get("bf16_tflops_sustained", 1700.0))
         nc = desc["tile_cols"]
         n_ct = -(-(N * P) // nc)
-        img_b = 192 * nc if desc["tile_rows"] == 64 else 384 * nc  # one stage image (layout 1: one B row per column)
+        one_row = desc["tile_rows"] == 64 or nc > 104              # one B row per column (row-doubled, CTA pairs)
+        img_b = 192 * nc if one_row else 384 * nc                  # one stage image
         images = T * n_ct * (-(-(3 * V) // 24)) * img_b            # stage images read per step
         shape = (desc["tile_rows"], nc)
         ratio = TC_DRAM_PER_IMAGE_BYTE.get(shape)
