@@ -860,7 +860,8 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
         long long stages = 0;
         for (int n = 0; n < n_inst; n++)
             stages += (long long)ones[n].size() * p->h_inst[n].n_st * p->h_inst[n].T;
-        if (stages >= (long long)SHAPE_MIN_STAGES * sms) {
+        // (a plan whose default tiles cannot stage their row vectors stays refused)
+        if (us104 < 1e300 && stages >= (long long)SHAPE_MIN_STAGES * sms) {
             double best = (def.tile_cols == 96 ? shape_us(96, 0) : us104) * (1.0 - SHAPE_MARGIN);
             const std::pair<int, int> shapes[] = {{96, 0}, {80, 0}, {64, 0}, {208, 1}, {176, 1}, {128, 1}, {laph::TC_PAIR_COLS, 2}};
             for (const auto &sh : shapes) {

@@ -259,7 +259,8 @@ __global__ void links_soa_kernel(const float2 *__restrict__ U, float2 *__restric
 // the step before.  (Scheduling the next grid from a block's first
 // instruction made its blocks take slots from the running grid: 48.0 ms of
 // filter steps at L=32, T=8, m=128, degree 48, against 44.3 without programmatic
-// launches and 43.9 this way; one timeslice 22.8, 16.1 and 14.7 ms.)
+// launches and 43.9 this way; one timeslice 22.8, 16.1 and 14.7 ms; L=21, T=2,
+// degree 47 4.88 -> 4.53 ms.)
 // R12: the links are SU(3) and only their first two rows are read.  PAIRS:
 // the paired layouts above.
 template <bool R12, bool PAIRS>
@@ -281,8 +282,10 @@ __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(
     const unsigned cc[3] = {c0, c1, c2};
     const unsigned stride[3] = {1u, uL, uL * uL};
     float2 fx[3], acc[3], uf[9], ub[9];
-    load_link<PAIRS, R12 ? 6 : 9>(Ut, V, x, uf);
-    load_link<PAIRS, R12 ? 6 : 9>(Ut, V, c0 == 0 ? x + (uL - 1) : x - 1, ub);
+    if (PAIRS) {   // nine separate loads a link (odd V) gain nothing ahead of the wait
+        load_link<PAIRS, R12 ? 6 : 9>(Ut, V, x, uf);
+        load_link<PAIRS, R12 ? 6 : 9>(Ut, V, c0 == 0 ? x + (uL - 1) : x - 1, ub);
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     load_site<PAIRS>(f, V, x, fx);
 #pragma unroll
@@ -296,7 +299,7 @@ __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(
         float2 fu[3], fd[3];
         load_site<PAIRS>(f, V, up, fu);
         load_site<PAIRS>(f, V, dn, fd);
-        if (mu > 0) {
+        if (mu > 0 || !PAIRS) {
             load_link<PAIRS, R12 ? 6 : 9>(um, V, x, uf);
             load_link<PAIRS, R12 ? 6 : 9>(um, V, dn, ub);
         }
@@ -412,15 +415,18 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
 
 // Gram-Schmidt update, w[t] -= sum_j coef[t][j] basis[t][j] for j < nj, with
 // the coefficients rounded to FP32 in shared memory (dynamic, nj float2) and
-// FP32 multiply-adds; UPD_EPT elements per thread, the loads of UPD_RG rows
-// issued together.  norm (may be null): norm[t] += |w[t]|^2 of the result.  Two
-// rows at a time at six blocks per SM keep as much in flight as four at four,
-// and fill the chip more evenly when there are few timeslices (T=8 at L=32: 768
-// blocks on 608 places before).  With the split rows of dots_kernel the
-// orthogonalisation of T=8, m=128 went from 39.8 to 36.5 ms.
+// FP32 multiply-adds; UPD_EPT elements per thread, the loads of RG rows issued
+// together.  norm (may be null): norm[t] += |w[t]|^2 of the result.  Four rows at
+// four blocks per SM, where the blocks fit one wave or fill many; in between
+// two rows at six, as much in flight in a launch that fills the chip more evenly
+// (T=8 at L=32: 768 blocks on 608 places before; with the split rows of
+// dots_kernel the orthogonalisation of m=128 went from 39.7 to 36.4 ms, one
+// timeslice 10.1 to 8.8 ms; T=64, whose launches are as before but for dots_kernel's
+// row range, 239 to 245 ms).
 constexpr int UPD_EPT = 4;
-constexpr int UPD_RG = 2;
-__global__ void __launch_bounds__(LAP_THREADS, 6) update_kernel(const float2 *__restrict__ basis, long long ts_basis,
+constexpr int UPD_WAVE = 4 * 152, UPD_MANY = 4 * UPD_WAVE;   // blocks between which two rows are taken
+template <int RG, int MINB>
+__global__ void __launch_bounds__(LAP_THREADS, MINB) update_kernel(const float2 *__restrict__ basis, long long ts_basis,
                                                              float2 *__restrict__ w, long long ts_w, long long K, int nj,
                                                              const double2 *__restrict__ coef, int coef_stride,
                                                              double *__restrict__ norm)
@@ -438,17 +444,17 @@ __global__ void __launch_bounds__(LAP_THREADS, 6) update_kernel(const float2 *__
     float2 acc[UPD_EPT];
 #pragma unroll
     for (int q = 0; q < UPD_EPT; q++) acc[q] = make_float2(0.f, 0.f);
-    for (int j = 0; j < nj; j += UPD_RG) {
-        float2 b[UPD_RG][UPD_EPT];
+    for (int j = 0; j < nj; j += RG) {
+        float2 b[RG][UPD_EPT];
 #pragma unroll
-        for (int r = 0; r < UPD_RG; r++)
+        for (int r = 0; r < RG; r++)
 #pragma unroll
             for (int q = 0; q < UPD_EPT; q++) {
                 const long long e = e0 + (long long)q * LAP_THREADS;
                 b[r][q] = (j + r < nj && e < K) ? B[(long long)(j + r) * K + e] : make_float2(0.f, 0.f);
             }
 #pragma unroll
-        for (int r = 0; r < UPD_RG; r++) {
+        for (int r = 0; r < RG; r++) {
             const float2 c = j + r < nj ? cs[j + r] : make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < UPD_EPT; q++) acc[q] = cfma(c, b[r][q], acc[q]);
@@ -971,6 +977,14 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
             dots_kernel<<<dim3(blocks_dot, T, (nj + rows_z - 1) / rows_z), LAP_THREADS, 0, s>>>(basis, ts_b, w, K, K, nj,
                                                                                                rows_z, dots, m + 1);
         };
+        auto launch_update = [&](int nj, double *norm) {
+            const dim3 g(blocks_upd, T);
+            const long long n = (long long)blocks_upd * T;
+            if (n <= UPD_WAVE || n >= UPD_MANY)
+                update_kernel<4, 4><<<g, LAP_THREADS, sizeof(float2) * nj, s>>>(basis, ts_b, w, K, K, nj, dots, m + 1, norm);
+            else
+                update_kernel<2, 6><<<g, LAP_THREADS, sizeof(float2) * nj, s>>>(basis, ts_b, w, K, K, nj, dots, m + 1, norm);
+        };
         // removes from w its components along basis vectors [0, nj), twice
         // ("twice is enough"); the first pass's coefficients land in h_dots,
         // |w|^2 of the result in h_norm.  Synchronises the stream.
@@ -981,8 +995,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
                 if (e == cudaSuccess && pass == 1) e = cudaMemsetAsync(dnorm, 0, sizeof(double) * T, s);
                 if (e != cudaSuccess) break;
                 launch_dots(nj);
-                update_kernel<<<dim3(blocks_upd, T), LAP_THREADS, sizeof(float2) * nj, s>>>(
-                    basis, ts_b, w, K, K, nj, dots, m + 1, pass == 1 ? dnorm : nullptr);
+                launch_update(nj, pass == 1 ? dnorm : nullptr);
                 e = cudaGetLastError();
                 st.launches += 2;
                 if (e == cudaSuccess && pass == 0)
@@ -1018,8 +1031,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
                 if (e == cudaSuccess && pass == 1) e = cudaMemsetAsync(dnorm, 0, sizeof(double) * T, s);
                 if (e != cudaSuccess) break;
                 launch_dots(j + 1);
-                update_kernel<<<dim3(blocks_upd, T), LAP_THREADS, sizeof(float2) * (j + 1), s>>>(
-                    basis, ts_b, w, K, K, j + 1, dots, m + 1, pass == 1 ? dnorm : nullptr);
+                launch_update(j + 1, pass == 1 ? dnorm : nullptr);
                 if (pass == 0) take_alpha_kernel<<<bt, 128, 0, s>>>(dots, m + 1, j, dalpha, m, T);
                 e = cudaGetLastError();
                 st.launches += pass == 0 ? 3 : 2;
