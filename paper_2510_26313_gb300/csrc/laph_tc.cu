@@ -18,7 +18,8 @@
 // K stages (chunk_stages_b for tiles without meson rows, whose incoherent
 // sums tolerate a longer interval) into a second tensor-memory region of
 // FP32 running sums kept by CUDA cores with round-to-nearest.  A tile covers
-// one block of sites (at most sc_stages K stages); at its end the running
+// one block of sites (at most sc_stages K stages), or one drain interval where
+// a plan cuts a small batch into them; at its end the running
 // sums are stored as FP32 partials, and reduce_kernel adds the partials of
 // all site blocks of an output in FP64, in block order, scales them back and
 // writes the complex128 (or complex64) output.  At chunk boundaries the MMAs of the two column halves
@@ -27,7 +28,8 @@
 //
 // Tile: 128 rows x 104 complex columns by default (UMMA M = 128, N = 208, the
 // widest that fits; 96, 80 and 64 columns, and 64 rows x 208, 192, 176 or
-// 128 columns in the row-doubled layout, are the other shapes).  A K stage
+// 128 columns in the row-doubled layout, are the other shapes; pairs of CTAs
+// work 128 rows x 208 columns, tc_pair_kernel; the plan chooses).  A K stage
 // is one site block: TC_BS = 8 sites = 24 complex = 48 real K entries, three
 // MMA k-steps of 16.
 // Tensor memory (512 columns): ACC [0,N) | SUM [N,2N) | two A slots of 48
