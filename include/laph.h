@@ -468,7 +468,9 @@ LAPH_API int laph_plan_drain_sites(const laph_plan *plan, int *chunk_sites, int 
 LAPH_API int laph_plan_launches_per_execute(const laph_plan *plan, int *n);
 
 /* Overrides the site-chunk length (sites summed in FP32 before the FP64
- * reduction; 0 = default).  Must be called before execute. */
+ * reduction; 0 = default) of the executes launched after the call.  Changes
+ * values on the host only: executes already queued and captured graphs keep
+ * the interval they were launched with. */
 LAPH_API int laph_plan_set_chunk_sites(laph_plan *plan, int chunk_sites);
 
 LAPH_API int laph_plan_destroy(laph_plan *plan);

@@ -132,7 +132,6 @@ struct laph_plan {
     // tensor-core path: chunks of (instance, timeslice) units and their B-operand images
     laph::PsiUnit *d_units = nullptr;
     std::vector<laph::PsiUnit> h_units;
-    std::vector<TileDev> h_tiles;   // kept only when some unit is cut into drains (laph_plan_set_chunk_sites)
     int psi_group = laph::TC_PSI_GROUP;   // stages per job of the B-operand pass
     // laph_plan_execute_host: copy streams and per-chunk events, made on first use
     cudaStream_t h2d = nullptr, d2h = nullptr;
@@ -151,6 +150,14 @@ struct laph_plan {
         long long n_red_split;   // blocks of their reduction
     };
     std::vector<Chunk> chunks;
+    // where units are cut into drains: the same schedule with whole site blocks,
+    // for laph_plan_set_chunk_sites.  Its tiles and units follow the cut ones in
+    // d_tiles, d_units and h_units (tile0 and unit0 count from the start of
+    // those), so that the call changes host values only: an execute in flight and
+    // a captured graph keep the tables that their launches were made for.
+    std::vector<Chunk> whole_chunks;
+    long long whole_n_tiles = 0;
+    double whole_flops = 0.0;
     // schedule of the tensor-core path: timeslices per chunk (0: chunks filled by
     // bytes) and tile order within a timeslice (0: column tiles outer, 1: row
     // tiles outer); with LAPH_PLAN_AUTOTUNE the candidates' timings
@@ -664,8 +671,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
             }
         }
         p->h_units = units;
-        p->h_tiles.clear();
-        if (n_split > 0) p->h_tiles = tiles;
+        p->whole_chunks.clear();
         p->sched_per_chunk = pc;
         p->sched_order = tile_order;
     };
@@ -735,7 +741,24 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
                 }
             }
         }
-        if (best > 0 || p->psi_group != laph::TC_PSI_GROUP) emit_tables(pc, tile_order, best);
+        if (p->psi_group != laph::TC_PSI_GROUP) emit_tables(pc, tile_order, 0);
+        if (best == 0) return;
+        const std::vector<TileDev> whole_tiles = tiles;
+        const std::vector<laph::PsiUnit> whole_units = units;
+        std::vector<laph_plan::Chunk> whole = p->chunks;
+        const long long n_whole = p->n_tiles;
+        const double flops = p->mma_flops;
+        emit_tables(pc, tile_order, best);
+        for (laph_plan::Chunk &c : whole) {
+            c.unit0 += (int)units.size();
+            c.tile0 += (long long)tiles.size();
+        }
+        tiles.insert(tiles.end(), whole_tiles.begin(), whole_tiles.end());
+        units.insert(units.end(), whole_units.begin(), whole_units.end());
+        p->h_units = units;
+        p->whole_chunks = whole;
+        p->whole_n_tiles = n_whole;
+        p->whole_flops = flops;
     };
     // device copies of the tables and the workspace layout (tensor-core modes:
     // per-timeslice max |phi| bits and one tile counter per chunk, both cleared
@@ -943,67 +966,19 @@ int laph_plan_sum_sites(const laph_plan *plan, int *sum_sites, int *max_site_blo
     return LAPH_OK;
 }
 
-// Takes back the cut into drains (its tiles and partials are made for one drain
-// interval): the unit's tiles cover whole site blocks again.  The workspace
-// layout stays; whole site blocks need a part of it.
-static int merge_drains(laph_plan *plan)
-{
-    if (plan->h_tiles.empty()) return LAPH_OK;
-    std::vector<TileDev> tiles;
-    std::vector<laph::PsiUnit> units = plan->h_units;
-    std::vector<laph_plan::Chunk> chunks = plan->chunks;
-    double flops = 0.0;
-    const int terms = (plan->mode == LAPH_MODE_TC_F16X3 || plan->mode == LAPH_MODE_TC_BF16X3) ? 3 : 1;
-    for (laph_plan::Chunk &c : chunks) {
-        const long long tile0 = (long long)tiles.size();
-        std::vector<long long> part(plan->total_ts, 0);
-        std::vector<int> split(plan->total_ts, 0);
-        c.n_red = c.n_red_split = 0;
-        c.n_split = 0;
-        for (int u = c.unit0; u < c.unit0 + c.n_units; u++) {
-            const InstDev &d = plan->h_inst[units[u].inst];
-            const long long n_out = d.n_outB + d.n_outM;
-            part[d.ts_base + units[u].t] = units[u].part_off;
-            split[d.ts_base + units[u].t] = units[u].split;
-            units[u].split = 0;
-            units[u].red0 = c.n_red;
-            c.n_red += (n_out + laph::TC_RED_BLOCK - 1) / laph::TC_RED_BLOCK;
-        }
-        for (long long q = c.tile0; q < c.tile0 + c.n_tiles; q++) {
-            TileDev v = plan->h_tiles[q];
-            const InstDev &d = plan->h_inst[v.inst];
-            const int ts = d.ts_base + v.t;
-            if (split[ts]) {
-                if (v.s0 % d.sc_stages) continue;
-                v.nst = std::min(d.sc_stages, d.n_st - v.s0);
-                v.part_off = part[ts] + (long long)(v.s0 / d.sc_stages) * (d.n_outB + d.n_outM);
-            }
-            const int n_real =
-                plan->rows2 ? ((v.ncols + 15) & ~15) - v.cskip : 2 * ((v.ncols + 7) & ~7) - 2 * v.cskip;
-            flops += 2.0 * laph::TC_TR * (plan->rows2 == 2 ? 2 : 1) * n_real * (2 * laph::TC_KSTAGE) * terms * v.nst;
-            tiles.push_back(v);
-        }
-        c.tile0 = tile0;
-        c.n_tiles = (long long)tiles.size() - tile0;
-    }
-    CK(cudaMemcpy(plan->d_tiles, tiles.data(), sizeof(TileDev) * tiles.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(plan->d_units, units.data(), sizeof(laph::PsiUnit) * units.size(), cudaMemcpyHostToDevice));
-    plan->h_units = units;
-    plan->chunks = chunks;
-    plan->n_tiles = (long long)tiles.size();
-    plan->mma_flops = flops;
-    plan->h_tiles.clear();
-    return LAPH_OK;
-}
-
+// Where units are cut into drains of one interval, another interval takes the
+// cut back: the tables of whole site blocks, made with the plan, take over.  The
+// workspace layout stays; whole site blocks need a part of it.
 int laph_plan_set_chunk_sites(laph_plan *plan, int chunk_sites)
 {
     if (!plan || chunk_sites < 0 || chunk_sites > (1 << 24)) return LAPH_ERR_ARG;
     const bool tc = is_tc_mode(plan->mode);
     if (chunk_sites == 0) chunk_sites = tc ? TC_DEFAULT_CHUNK : SIMT_DEFAULT_CHUNK;
-    if (chunk_sites != plan->chunk_sites) {
-        const int rc = merge_drains(plan);
-        if (rc != LAPH_OK) return rc;
+    if (chunk_sites != plan->chunk_sites && !plan->whole_chunks.empty()) {
+        plan->chunks.swap(plan->whole_chunks);
+        plan->n_tiles = plan->whole_n_tiles;
+        plan->mma_flops = plan->whole_flops;
+        plan->whole_chunks.clear();
     }
     plan->chunk_sites = chunk_sites;
     return LAPH_OK;
