@@ -154,7 +154,7 @@ __device__ __forceinline__ void su3_third_row(float2 *u)
 // The orthogonalisation and Ritz kernels treat a vector as 3V elements in any
 // order; the final gather writes the caller's [V][3].
 template <bool PAIRS>
-__device__ __forceinline__ void load_site(const float2 *__restrict__ f, unsigned V, unsigned x, float2 v[3])
+__device__ __forceinline__ void load_site(const float2 *f, unsigned V, unsigned x, float2 v[3])
 {
     if (PAIRS) {
         const float4 p = reinterpret_cast<const float4 *>(f)[x];
@@ -168,7 +168,7 @@ __device__ __forceinline__ void load_site(const float2 *__restrict__ f, unsigned
 }
 
 template <bool PAIRS>
-__device__ __forceinline__ void store_site(float2 *__restrict__ o, unsigned V, unsigned x, const float2 v[3])
+__device__ __forceinline__ void store_site(float2 *o, unsigned V, unsigned x, const float2 v[3])
 {
     if (PAIRS) {
         reinterpret_cast<float4 *>(o)[x] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
@@ -261,12 +261,14 @@ __global__ void links_soa_kernel(const float2 *__restrict__ U, float2 *__restric
 // filter steps at L=32, T=8, m=128, degree 48, against 44.3 without programmatic
 // launches and 43.9 this way; one timeslice 22.8, 16.1 and 14.7 ms; L=21, T=2,
 // degree 47 4.88 -> 4.53 ms.)
+// The vectors carry no promise of being read-only or unaliased: the grid is
+// resident while its predecessor still writes `in`, so their loads have to stay
+// coherent and behind the wait (the links' may be read-only loads ahead of it).
 // R12: the links are SU(3) and only their first two rows are read.  PAIRS:
 // the paired layouts above.
 template <bool R12, bool PAIRS>
 __global__ void __launch_bounds__(LAP_SOA_THREADS, LAP_SOA_MINB) lap_soa_kernel(const float2 *__restrict__ Us,
-                                                              const float2 *__restrict__ in,
-                                                              const float2 *__restrict__ z, float2 *__restrict__ out,
+                                                              const float2 *in, const float2 *z, float2 *out,
                                                               int L, long long ts_in, long long ts_z, long long ts_out,
                                                               float a, float b, float c)
 {
