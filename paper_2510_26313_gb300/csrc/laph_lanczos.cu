@@ -353,7 +353,11 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
 // FP64 arithmetic runs per element.  Block z takes its share of the rows
 // (rows_z, a multiple of DOT_JC): the sums of different rows do not meet, and a
 // few timeslices alone are little more than one wave of blocks (T=8 at L=32:
-// 384 on 304 places).
+// 384 on 304 places).  The share is taken off the pointers and nj ahead of the
+// loop: with the range in the loop's bounds the kernel was slower by itself,
+// also where a block keeps all rows (orthogonalisation, m=128: T=64 244.9 ->
+// 238.1 ms, T=8 36.2 -> 35.0, one timeslice 8.4 -> 7.6; L=21, T=2, m=36 1.67 ->
+// 1.52).
 constexpr int DOT_EPT = 8;      // elements of w per thread
 constexpr int DOT_JC = 32;      // rows between flushes of the warp partials
 constexpr int DOT_RG = 4;       // rows whose loads are issued together
@@ -365,16 +369,18 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
     __shared__ float2 part[LAP_THREADS / 32][DOT_JC];
     const int t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long e0 = (long long)blockIdx.x * LAP_THREADS * DOT_EPT + threadIdx.x;
-    const float2 *B = basis + t * ts_basis;
+    const int jz = blockIdx.z * rows_z;
+    const float2 *B = basis + t * ts_basis + jz * K;
+    nj = min(nj - jz, rows_z);
+    dots += t * dots_stride + jz;
     float2 wv[DOT_EPT];
 #pragma unroll
     for (int q = 0; q < DOT_EPT; q++) {
         const long long e = e0 + (long long)q * LAP_THREADS;
         wv[q] = e < K ? w[t * ts_w + e] : make_float2(0.f, 0.f);
     }
-    const int j_end = min(nj, ((int)blockIdx.z + 1) * rows_z);
-    for (int j0 = blockIdx.z * rows_z; j0 < j_end; j0 += DOT_JC) {
-        const int jn = min(DOT_JC, j_end - j0);
+    for (int j0 = 0; j0 < nj; j0 += DOT_JC) {
+        const int jn = min(DOT_JC, nj - j0);
         for (int jj = 0; jj < jn; jj += DOT_RG) {
             float2 b[DOT_RG][DOT_EPT];
 #pragma unroll
@@ -408,8 +414,8 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
                 re += part[q][threadIdx.x].x;
                 im += part[q][threadIdx.x].y;
             }
-            atomicAdd(&dots[t * dots_stride + j0 + threadIdx.x].x, re);
-            atomicAdd(&dots[t * dots_stride + j0 + threadIdx.x].y, im);
+            atomicAdd(&dots[j0 + threadIdx.x].x, re);
+            atomicAdd(&dots[j0 + threadIdx.x].y, im);
         }
         __syncthreads();
     }
@@ -421,10 +427,9 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
 // together.  norm (may be null): norm[t] += |w[t]|^2 of the result.  Four rows at
 // four blocks per SM, where the blocks fit one wave or fill many; in between
 // two rows at six, as much in flight in a launch that fills the chip more evenly
-// (T=8 at L=32: 768 blocks on 608 places before; with the split rows of
-// dots_kernel the orthogonalisation of m=128 went from 39.7 to 36.4 ms, one
-// timeslice 10.1 to 8.8 ms; T=64, whose launches are as before but for dots_kernel's
-// row range, 239 to 245 ms).
+// (T=8 at L=32: 768 blocks on 608 places before; with the shared rows of
+// dots_kernel the orthogonalisation of m=128 went from 39.5 to 35.0 ms, one
+// timeslice 10.0 to 7.6 ms, T=64 238.5 to 238.1 ms).
 constexpr int UPD_EPT = 4;
 constexpr int UPD_WAVE = 4 * 152, UPD_MANY = 4 * UPD_WAVE;   // blocks between which two rows are taken
 template <int RG, int MINB>
