@@ -431,7 +431,8 @@ __global__ void __launch_bounds__(LAP_THREADS) dots_kernel(const float2 *__restr
 // dots_kernel the orthogonalisation of m=128 went from 39.5 to 35.0 ms, one
 // timeslice 10.0 to 7.6 ms, T=64 238.5 to 238.1 ms).
 constexpr int UPD_EPT = 4;
-constexpr int UPD_WAVE = 4 * 152, UPD_MANY = 4 * UPD_WAVE;   // blocks between which two rows are taken
+constexpr int UPD_WAVE = 4, UPD_MANY = 16;   // blocks per SM between which two rows are taken
+constexpr int DOT_BLOCKS = 6;                // blocks per SM up to which dots_kernel shares its rows out
 template <int RG, int MINB>
 __global__ void __launch_bounds__(LAP_THREADS, MINB) update_kernel(const float2 *__restrict__ basis, long long ts_basis,
                                                              float2 *__restrict__ w, long long ts_w, long long K, int nj,
@@ -878,9 +879,10 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
     // timeslice, stay in L2 across its d steps: groups filling about 70% of the
     // L2 (measured at L = 32, T = 64 on GB300: 8 timeslices, 88 MB, take 0.71x
     // the time of one group of all 64; 16 timeslices overflow it)
-    int tg = prm->ts_group, dev = 0, l2 = 0;
+    int tg = prm->ts_group, dev = 0, l2 = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
         l2 = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) sms = 0;
     if (tg == 0) tg = (int)std::max<long long>(1, (long long)(0.7 * l2) / (8 * 42 * V));
     tg = std::min(tg, T);
     // SU(3) links can be read as two rows (the third rebuilt), 144 instead of
@@ -977,7 +979,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
         };
         // inner products of w with basis vectors [0, nj), the rows shared out until there are a few waves of blocks
         auto launch_dots = [&](int nj) {
-            const long long want = 6LL * 152, have = (long long)blocks_dot * T;
+            const long long want = (long long)DOT_BLOCKS * sms, have = (long long)blocks_dot * T;
             const int chunks = (nj + DOT_JC - 1) / DOT_JC;
             const int nz = (int)std::max(1LL, std::min<long long>(chunks, (want + have - 1) / have));
             const int rows_z = (chunks + nz - 1) / nz * DOT_JC;
@@ -987,7 +989,7 @@ int laph_lanczos(const void *U, int L, int T, int n_ev, const laph_lanczos_param
         auto launch_update = [&](int nj, double *norm) {
             const dim3 g(blocks_upd, T);
             const long long n = (long long)blocks_upd * T;
-            if (n <= UPD_WAVE || n >= UPD_MANY)
+            if (n <= (long long)UPD_WAVE * sms || n >= (long long)UPD_MANY * sms)
                 update_kernel<4, 4><<<g, LAP_THREADS, sizeof(float2) * nj, s>>>(basis, ts_b, w, K, K, nj, dots, m + 1, norm);
             else
                 update_kernel<2, 6><<<g, LAP_THREADS, sizeof(float2) * nj, s>>>(basis, ts_b, w, K, K, nj, dots, m + 1, norm);
