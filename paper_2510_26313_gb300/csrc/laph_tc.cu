@@ -358,12 +358,13 @@ __device__ __noinline__ bool warp_wait_slow(Shared *S, int *status, int lane, ui
 }
 
 // Bounded wait that ignores the abort flag: used at exit to let the bulk
-// copies a warp issued land before the CTA's shared memory is released.
+// copies and MMAs a warp issued complete before shared and tensor memory are
+// released.
 __device__ __noinline__ void drain_wait(Shared *S, int *status, int lane, uint64_t *bar, uint32_t parity)
 {
     const long long t0 = clock64();
     while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
-        if (clock64() - t0 > WAIT_LIMIT) {
+        if (__shfl_sync(0xffffffffu, (int)(clock64() - t0 > WAIT_LIMIT), 0)) {
             if (lane == 0) {
                 *(volatile int *)&S->abort = 1;
                 atomicOr(status, STATUS_TIMEOUT);
@@ -810,6 +811,7 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
                     break;
                 }
                 tc_fence_after();
+                issued = true;
                 const uint32_t a_hi = tmem + A_COL + (uint32_t)ra.slot * A_SLOT_COLS, a_lo = a_hi + A_LO;
                 // descriptor start addresses advance one atom column (in units of 16 bytes) per k-step
                 const uint64_t dhi = desc_sw32(smem_u32(smem + rs.slot * kp.stage_bytes)) + bskip;
@@ -860,7 +862,6 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
                 if (lane == 0) {
                     // one commit frees the stage buffer (loader) and the A slot (producers)
                     mma_commit(&S->empty[rs.slot]);
-                    issued = true;
                 }
                 __syncwarp();
                 cs = chunk_end ? 0 : cs + 1;
@@ -868,10 +869,10 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
                 ra.next(2);
             }
         }
-        // every issued MMA has completed before tensor memory is released
+        // every issued MMA has completed before tensor memory is released, after an abort too
         if (lane == 0 && issued) mma_commit(&S->done);
         __syncwarp();
-        if (__shfl_sync(0xffffffffu, issued ? 1 : 0, 0)) warp_wait(c, &S->done, 0u);
+        if (issued) drain_wait(S, kp.status, lane, &S->done, 0u);
     }
 
     __syncthreads();
@@ -1326,23 +1327,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
                 ra.next(2);
             }
         }
-        // every issued MMA has completed before tensor memory is released
+        // every issued MMA has completed before either CTA releases shared or
+        // tensor memory, after an abort too
         if (lane == 0) commit_pair(&S->done);
         __syncwarp();
-        warp_wait(c, &S->done, 0u);
+        drain_wait(S, kp.status, lane, &S->done, 0u);
     } else {
-        // CTA 1's idle MMA warp follows the tiles, so that its wait for the last
-        // commit is a short one
+        // CTA 1's idle MMA warp follows the tiles (it is one of their readers)
         Ring rt{0, 0};
         bool ok = true;
         while (ok && next_tile_pair(c, rt, ok) >= 0) {
         }
-        warp_wait(c, &S->done, 0u);
     }
 
     __syncthreads();
     cluster_sync_all();   // neither CTA leaves or frees tensor memory while the other may reach into it
     if (warp == WARP_MMA) {
+        // the last commit has been made: its arrival here is the last one from CTA 0
+        if (rank) drain_wait(S, kp.status, lane, &S->done, 0u);
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }

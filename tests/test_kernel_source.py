@@ -2,6 +2,8 @@
 import os
 import re
 
+import pytest
+
 from helpers import ROOT
 
 CSRC = os.path.join(ROOT, "paper_2510_26313_gb300", "csrc")
@@ -34,3 +36,17 @@ def test_filter_vectors_are_not_promised_read_only():
     assert "__ldg" not in body(src, "load_site(")
     # the first access to a vector comes after the wait
     assert k.index("griddepcontrol.wait") < k.index("load_site<")
+
+
+@pytest.mark.parametrize("kernel", ["tc_kernel(", "tc_pair_kernel("])
+def test_exit_waits_for_the_last_mma_ignore_the_abort_flag(kernel):
+    """The wait for the last commit stands between the MMAs and the release of shared and tensor memory (in a pair of
+    CTAs also the other CTA's): after an abort it must not return early, as the waits of the roles do."""
+    k = body(source("laph_tc.cu"), kernel)
+    waits = re.findall(r"(\w+)\([^;]*&S->done, 0u\)", k)
+    assert waits and set(waits) == {"drain_wait"}
+    assert k.rindex("&S->done, 0u") < k.rindex("dealloc")
+    if "pair" in kernel:   # CTA 0 waits before the CTAs meet, CTA 1 for the commit's arrival after that
+        assert len(waits) == 2
+        first, last = [m.start() for m in re.finditer(r"&S->done, 0u", k)]
+        assert first < k.rindex("cluster_sync_all()") < last
