@@ -991,6 +991,7 @@ static laph::TcConfig tc_config(const laph_plan *p)
     cfg.terms = (p->mode == LAPH_MODE_TC_F16X3 || p->mode == LAPH_MODE_TC_BF16X3) ? 3 : 1;
     cfg.chunk_sites = p->chunk_sites;
     cfg.chunk_sites_b = p->chunk_sites_b;
+    cfg.psi_bytes = p->off_part - p->off_psi;
     cfg.ncols = p->tile_cols;
     cfg.rows2 = p->rows2;
     cfg.grid = p->grid;

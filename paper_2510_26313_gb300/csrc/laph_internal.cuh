@@ -201,6 +201,7 @@ struct TcConfig {
     int chunk_sites_b; // the same for tiles without meson rows
     int grid;          // persistent CTAs
     int max_staged;    // largest number of staged row vectors (nv) of any tile
+    size_t psi_bytes;  // size of the stage-image buffer
     int debug_stall;   // test hook
 };
 constexpr int TC_TR = 128;   // tile rows (UMMA M)

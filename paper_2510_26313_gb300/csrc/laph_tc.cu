@@ -65,6 +65,7 @@
 // STATUS_TIMEOUT, raises a shared abort flag and all roles return.
 #include <algorithm>
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -144,6 +145,7 @@ struct Shared {
     uint64_t a_full[2];
     uint64_t acc_full[2], acc_empty[2];   // per column half of the accumulator
     uint64_t done;
+    uint32_t n_issued[2];                 // CTA pairs, in CTA 0: stages whose copies either loader issued
     uint32_t tmem_base;
     int abort;
 };
@@ -163,17 +165,29 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 }
 
 // Tests the phase with the given parity for completion; the warp may be
-// suspended for a system-dependent time while it is incomplete.
+// suspended for a system-dependent time while it is incomplete.  W_CTA acquires
+// at CTA scope; W_RELAXED and W_CLUSTER observe at cluster scope, without and with
+// acquire (CTA pairs).
+enum { W_CTA, W_RELAXED, W_CLUSTER };
+template <int KIND = W_CTA>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
+#define LAPH_TRY_WAIT(sem)                                                              \
+    asm volatile(                                                                       \
+        "{\n\t.reg .pred p;\n\t"                                                        \
+        "mbarrier.try_wait.parity" sem ".shared::cta.b64 p, [%1], %2;\n\t"              \
+        "selp.u32 %0, 1, 0, p;\n\t}"                                                    \
+        : "=r"(ok)                                                                      \
+        : "r"(smem_u32(bar)), "r"(parity)                                               \
+        : "memory")
+    if (KIND == W_RELAXED)
+        LAPH_TRY_WAIT(".relaxed.cluster");
+    else if (KIND == W_CLUSTER)
+        LAPH_TRY_WAIT(".acquire.cluster");
+    else
+        LAPH_TRY_WAIT("");
+#undef LAPH_TRY_WAIT
     return ok != 0;
 }
 
@@ -338,11 +352,12 @@ struct Ctx {
 // Slow path of a warp-wide bounded wait.  Between the try_waits (each may
 // suspend the warp for a while) the abort flag and the time limit are
 // checked.
+template <int KIND>
 __device__ __noinline__ bool warp_wait_slow(Shared *S, int *status, int lane, uint64_t *bar, uint32_t parity)
 {
     const long long t0 = clock64();
     while (true) {
-        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__all_sync(0xffffffffu, mbar_try_wait<KIND>(bar, parity))) return true;
         const int ab = *(volatile int *)&S->abort;
         if (__any_sync(0xffffffffu, ab != 0)) return false;
         int expired = (clock64() - t0) > WAIT_LIMIT;
@@ -375,10 +390,11 @@ __device__ __noinline__ void drain_wait(Shared *S, int *status, int lane, uint64
 }
 
 // Warp-wide bounded wait (every lane calls it; the result is warp-uniform).
+template <int KIND = W_CTA>
 __device__ __forceinline__ bool warp_wait(const Ctx c, uint64_t *bar, uint32_t parity)
 {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return warp_wait_slow(c.S, c.status, c.lane, bar, parity);
+    if (__all_sync(0xffffffffu, mbar_try_wait<KIND>(bar, parity))) return true;
+    return warp_wait_slow<KIND>(c.S, c.status, c.lane, bar, parity);
 }
 
 // Ring position: slot index and the parity of its current phase.
@@ -897,15 +913,16 @@ __global__ void __launch_bounds__(Roles<RD>::NTHREADS, 1) tc_kernel(const KParam
 // Roles as in tc_kernel (column-doubled warp counts).  CTA 0's loader claims
 // the pair's tiles and hands them to both CTAs; its MMA warp issues for both,
 // and its commits arrive on the barriers of both (multicast).  The producers'
-// and epilogue warps' arrivals for the MMA warp, and every reader's for the
-// tile ring, go to CTA 0.  The accumulator is drained whole: all its columns
-// are committed together, and the next chunk starts when both CTAs have
-// drained them.
+// and epilogue warps' arrivals for the MMA warp, every reader's for the tile
+// ring, and the completion of CTA 1's half of B go to CTA 0.  The accumulator is
+// drained whole: all its columns are committed together, and the next chunk
+// starts when both CTAs have drained them.
 //
 // The half-size B stage leaves a ring of four buffers where tc_kernel's is
 // three deep (more than about 80 row vectors per tile), which is what it is
-// used for: L=48, N=128, 33 momenta, one timeslice: contraction 68.2 -> 66.0 ms,
-// B-operand pass 3.65 -> 2.60 ms.  With four buffers on both sides the two run
+// used for: L=48, N=128, 33 momenta, one timeslice: contraction 70.3 -> 66.7 ms,
+// with its B-operand pass and the rest 75.8 -> 71.0 ms; L=24, N=100, two
+// timeslices 10.1 -> 8.7.  With four buffers on both sides the two run
 // alike (three fields, L=32, N=64: 7.73 against 7.75 ms): the period of a stage
 // is set by the producers and the power limit, not by the B operand.
 constexpr int PAIR_NC = TC_PAIR_COLS;
@@ -915,6 +932,10 @@ constexpr int PAIR_ATOM_BYTES = PAIR_B_BYTES / KSTEPS;              // one k-ste
 constexpr int PAIR_READERS = (N_AWARPS + 8 + 1) + (N_AWARPS + 8 + 2);
 static_assert(PAIR_NC % 16 == 0 && 2 * PAIR_NC <= (int)A_COL, "tile width within the tensor-memory budget");
 static_assert(2 * PAIR_HALF_BYTES == tc_stage_bytes(PAIR_NC, true), "stage image size");
+// Tensor map over the stage images: rows of MAP_ROW bytes (192 elements of 8
+// bytes), half an image is one box of whole rows.
+constexpr int MAP_ROW = 1536, MAP_BOX = PAIR_HALF_BYTES / MAP_ROW;
+static_assert(PAIR_HALF_BYTES % MAP_ROW == 0 && MAP_ROW / 8 <= 256 && MAP_BOX <= 256, "box limits");
 
 __device__ __forceinline__ uint32_t cta_rank()
 {
@@ -936,13 +957,15 @@ __device__ __forceinline__ uint32_t peer_addr(const void *p, uint32_t rank)
     return a;
 }
 
-// Arrival on a barrier of either CTA.  The plain form orders what these
-// arrivals order: tensor-memory accesses (with the tcgen05 fences) and the use
-// of a ring slot.  Cluster-scope release and acquire, which wait for memory
-// traffic, are kept for the tile ring's entries, once per tile.
+// Arrivals between the CTAs, at cluster scope like the waits for them.  Relaxed
+// ones hand over tensor memory, whose accesses the tcgen05 fences around them
+// order.  Release and acquire, which wait for memory traffic (on every barrier
+// they made a stage take 1.11 us instead of 0.74), hand over the tile ring's
+// entries, once per tile.  CTA 1's half of B needs neither: its copies complete
+// on the stage's data barrier in CTA 0.
 __device__ __forceinline__ void mbar_arrive_at(uint32_t addr)
 {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t addr)
@@ -950,41 +973,32 @@ __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t addr)
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// warp_wait with acquire at cluster scope: for barriers that the other CTA's
-// threads arrive on.
-__device__ __forceinline__ bool warp_wait_cluster(const Ctx c, uint64_t *bar, uint32_t parity)
-{
-    if (!__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) {
-        if (!warp_wait_slow(c.S, c.status, c.lane, bar, parity)) return false;
-        mbar_try_wait_cluster(bar, parity);   // the phase is complete: acquires at cluster scope
-    }
-    return true;
-}
-
 __device__ __forceinline__ int next_tile_pair(const Ctx c, Ring &rt, bool &ok)
 {
-    if (!warp_wait_cluster(c, &c.S->tfull[rt.slot], rt.phase)) {
+    if (!warp_wait<W_CLUSTER>(c, &c.S->tfull[rt.slot], rt.phase)) {
         ok = false;
         return -1;
     }
     const int t = *(volatile int *)&c.S->tile_ring[rt.slot];
     __syncwarp();
-    if (c.lane == 0) mbar_arrive_at(peer_addr(&c.S->tempty[rt.slot], 0));
+    if (c.lane == 0) mbar_arrive_release_cluster(peer_addr(&c.S->tempty[rt.slot], 0));
     rt.next(TRING);
     return t;
+}
+
+// CTA 1's half of a B stage: the data barrier in CTA 0 is armed from here too, and
+// the copy (a tile of the tensor map over the stage images; the form that may
+// complete on the other CTA's barrier) completes on it.
+__device__ __forceinline__ void tma_b1(void *dst, const CUtensorMap *map, int row, uint32_t bar0)
+{
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar0),
+                 "r"(PAIR_HALF_BYTES)
+                 : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, "
+        "%3}], [%4];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(0), "r"(row), "r"(bar0)
+        : "memory");
 }
 
 // M = 256 over the pair: 128 rows in each CTA.
@@ -1016,7 +1030,7 @@ __device__ __forceinline__ void commit_pair(uint64_t *bar)
 }
 
 template <int ELEM, int TERMS>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREADS, 1) tc_pair_kernel(const KParams kp)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREADS, 1) tc_pair_kernel(const KParams kp, const __grid_constant__ CUtensorMap bmap)
 {
     using R = Roles<false>;
     constexpr int WARP_LOAD = R::WARP_LOAD, WARP_MMA = R::WARP_MMA;
@@ -1031,8 +1045,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; s++) {
-            mbar_init(&S->full[s], 1);
-            mbar_init(&S->full[NS + s], 1);
+            mbar_init(&S->full[s], rank ? 1 : 2);        // armed by the loader, in CTA 0 by both
+            mbar_init(&S->full[NS + s], rank ? 1 : 2);
             mbar_init(&S->empty[s], 1);
         }
         for (int s = 0; s < TRING; s++) {
@@ -1066,7 +1080,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
         while (ok) {
             int tile = 0;
             if (rank == 0) {
-                if (!warp_wait(c, &S->tempty[rt.slot], rt.phase ^ 1u)) break;
+                if (!warp_wait<W_CLUSTER>(c, &S->tempty[rt.slot], rt.phase ^ 1u)) break;
                 if (lane == 0) {
                     tile = (int)atomicAdd(kp.counter, 1u);
                     if (tile >= kp.n_tiles) tile = -1;
@@ -1086,21 +1100,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
             const InstDev &I = kp.insts[td.inst];
             const int nst = td.nst;
             const uint32_t bytesA = td.nv * SLOT_BYTES, bytesW = td.nw * SLOT_BYTES;
-            const uint8_t *bsrc = kp.psi + td.psi_off + (long long)td.s0 * (2 * PAIR_HALF_BYTES) + rank * PAIR_HALF_BYTES;
+            // B: CTA 0's half of a stage image by a bulk copy, CTA 1's as a box of the tensor map
+            const uint8_t *bsrc = kp.psi + td.psi_off + (long long)td.s0 * (2 * PAIR_HALF_BYTES);
+            const int brow = (int)(td.psi_off / MAP_ROW) + (2 * td.s0 + 1) * MAP_BOX;
             const long long blk0 = ((long long)td.t * I.nblk + td.s0) * I.N;
             const float2 *asrc = I.phi_blk + (blk0 + td.v_lo) * TC_SLOT;
             const float2 *wsrc = I.blk_v + (blk0 + td.w_lo) * TC_SLOT;
             const long long astep = (long long)I.N * TC_SLOT;
             for (int st = 0; st < nst; st++) {
-                if (!warp_wait(c, &S->empty[rs.slot], rs.phase ^ 1u)) {
+                if (!warp_wait<W_RELAXED>(c, &S->empty[rs.slot], rs.phase ^ 1u)) {
                     ok = false;
                     break;
                 }
                 if (lane == 0) {
                     uint8_t *buf = smem + rs.slot * kp.stage_bytes;
                     uint64_t *fb = &S->full[rf.slot];
-                    mbar_arrive_expect_tx(fb, PAIR_HALF_BYTES + bytesA + bytesW);
-                    bulk_g2s(buf, bsrc + (long long)st * (2 * PAIR_HALF_BYTES), PAIR_HALF_BYTES, fb);
+                    mbar_arrive_expect_tx(fb, (rank ? 0 : PAIR_HALF_BYTES) + bytesA + bytesW);
+                    if (rank)
+                        tma_b1(buf, &bmap, brow + 2 * st * MAP_BOX, peer_addr(fb, 0));
+                    else
+                        bulk_g2s(buf, bsrc + (long long)st * (2 * PAIR_HALF_BYTES), PAIR_HALF_BYTES, fb);
                     bulk_g2s(buf + PAIR_HALF_BYTES, asrc + st * astep, bytesA, fb);
                     if (bytesW) bulk_g2s(buf + PAIR_HALF_BYTES + bytesA, wsrc + st * astep, bytesW, fb);
                 }
@@ -1110,8 +1129,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
                 n_issued++;
             }
         }
-        for (uint32_t k = n_issued > (uint32_t)NS ? n_issued - NS : 0; k < n_issued; k++)
-            drain_wait(S, kp.status, lane, &S->full[k % (2 * NS)], (k / (2 * NS)) & 1u);
+        if (rank)
+            for (uint32_t k = n_issued > (uint32_t)NS ? n_issued - NS : 0; k < n_issued; k++)
+                drain_wait(S, kp.status, lane, &S->full[k % (2 * NS)], (k / (2 * NS)) & 1u);
+        if (lane == 0)
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(&S->n_issued[rank], 0)), "r"(n_issued)
+                         : "memory");
     } else if (warp < N_AWARPS) {
         // ---------------------------------------------------------- A producers
         const int quad = warp & 3, half = (warp >> 2) & 1, grp = warp >> 3;
@@ -1166,7 +1189,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
                     a_quarter<ELEM, 0>(kind, buf + off_u, buf + off_v, hi, lo);
                 else
                     a_quarter<ELEM, 3>(kind, buf + off_u, buf + off_v, hi, lo);
-                if (!warp_wait(c, &S->empty[s2], ph2)) {
+                if (!warp_wait<W_RELAXED>(c, &S->empty[s2], ph2)) {
                     ok = false;
                     break;
                 }
@@ -1177,7 +1200,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
                 __syncwarp();
                 const bool skip = kp.debug_stall && !stalled && blockIdx.x == 0 && warp == 0;
                 if (skip) stalled = true;
-                if (lane == 0 && !skip) mbar_arrive_at(a_full0);
+                if (lane == 0 && !skip) {
+                    if (rank == 0)
+                        mbar_arrive(&S->a_full[grp]);
+                    else
+                        mbar_arrive_at(a_full0);
+                }
                 s += 2;
                 if (s >= NS) s -= NS;
                 sf += 2;
@@ -1210,7 +1238,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
             const int cs = td.row0 >= I.mes_rows ? kp.chunk_stages_b : kp.chunk_stages;
             const int n_ch = (td.nst + cs - 1) / cs;
             for (int ch = 0; ch < n_ch; ch++) {
-                if (!warp_wait(c, &S->acc_full[0], g & 1u)) {
+                if (!warp_wait<W_RELAXED>(c, &S->acc_full[0], g & 1u)) {
                     ok = false;
                     break;
                 }
@@ -1291,11 +1319,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
             int cs = 0;   // stage within the current accumulation chunk
             for (int st = 0; st < nst; st++) {
                 const bool chunk_end = cs + 1 == chunk || st + 1 == nst;
-                if (cs == 0 && !warp_wait(c, &S->acc_empty[0], (g & 1u) ^ 1u)) {
+                if (cs == 0 && !warp_wait<W_RELAXED>(c, &S->acc_empty[0], (g & 1u) ^ 1u)) {
                     ok = false;
                     break;
                 }
-                if (!warp_wait(c, &S->a_full[ra.slot], ra.phase)) {
+                // both CTAs' A rows are in place, and both halves of B: CTA 0's producers waited for them on CTA 0's
+                // data barrier before their release-arrives
+                if (!warp_wait<W_CLUSTER>(c, &S->a_full[ra.slot], ra.phase)) {
                     ok = false;
                     break;
                 }
@@ -1341,7 +1371,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Roles<false>::NTHREA
     }
 
     __syncthreads();
-    cluster_sync_all();   // neither CTA leaves or frees tensor memory while the other may reach into it
+    // neither CTA leaves or frees tensor memory while the other may reach into it.
+    // CTA 0's data barriers count both CTAs' copies: the last ones land first (after
+    // an abort nobody waited for them, and one loader may have issued stages that
+    // the other did not: the arming that is missing is made up for)
+    cluster_sync_all();
+    if (rank == 0 && warp == WARP_LOAD) {
+        const uint32_t n0 = *(volatile uint32_t *)&S->n_issued[0], n1 = *(volatile uint32_t *)&S->n_issued[1];
+        const uint32_t n = max(n0, n1);
+        if (lane == 0)
+            for (uint32_t k = min(n0, n1); k < n; k++) mbar_arrive(&S->full[k % (2 * NS)]);
+        __syncwarp();
+        for (uint32_t k = n > (uint32_t)NS ? n - NS : 0; k < n; k++)
+            drain_wait(S, kp.status, lane, &S->full[k % (2 * NS)], (k / (2 * NS)) & 1u);
+    }
+    __syncwarp();
+    cluster_sync_all();
     if (warp == WARP_MMA) {
         // the last commit has been made: its arrival here is the last one from CTA 0
         if (rank) drain_wait(S, kp.status, lane, &S->done, 0u);
@@ -1700,6 +1745,27 @@ int pair_ring_depth(int max_staged)
     return 0;
 }
 
+// Tensor map of the stage images at psi (see tma_b1).
+cudaError_t map_images(const uint8_t *psi, size_t bytes, CUtensorMap *map)
+{
+    using Encode = decltype(&cuTensorMapEncodeTiled);
+    static const Encode encode = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return (Encode)f;
+    }();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dim[2] = {MAP_ROW / 8, bytes / MAP_ROW}, stride[1] = {MAP_ROW};
+    const cuuint32_t box[2] = {MAP_ROW / 8, MAP_BOX}, one[2] = {1, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<uint8_t *>(psi), dim, stride, box, one,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 template <int ELEM, int TERMS>
 cudaError_t launch_pair(const InstDev *d_inst, const TileDev *d_tiles, long long n_tiles, const unsigned *maxbits,
                         const uint8_t *psi, float2 *part, unsigned *counter, const TcConfig &cfg, int *status,
@@ -1712,11 +1778,13 @@ cudaError_t launch_pair(const InstDev *d_inst, const TileDev *d_tiles, long long
     kp.ns = pair_ring_depth(cfg.max_staged);
     if (!kp.ns) return cudaErrorNotSupported;
     const int smem = smem_for(kp.ns, kp.stage_bytes);
-    const cudaError_t e =
-        cudaFuncSetAttribute(tc_pair_kernel<ELEM, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    CUtensorMap bmap;
+    cudaError_t e = map_images(psi, cfg.psi_bytes, &bmap);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc_pair_kernel<ELEM, TERMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const long long pairs = std::min<long long>(std::max(1, cfg.grid / 2), n_tiles);
-    tc_pair_kernel<ELEM, TERMS><<<(unsigned)(2 * pairs), Roles<false>::NTHREADS, smem, s>>>(kp);
+    tc_pair_kernel<ELEM, TERMS><<<(unsigned)(2 * pairs), Roles<false>::NTHREADS, smem, s>>>(kp, bmap);
     return cudaGetLastError();
 }
 

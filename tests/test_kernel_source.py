@@ -50,3 +50,16 @@ def test_exit_waits_for_the_last_mma_ignore_the_abort_flag(kernel):
         assert len(waits) == 2
         first, last = [m.start() for m in re.finditer(r"&S->done, 0u", k)]
         assert first < k.rindex("cluster_sync_all()") < last
+
+
+def test_arrivals_between_the_ctas_of_a_pair_name_the_cluster_scope():
+    """Without a scope an mbarrier operation's is the CTA, which does not order it with the other CTA's.  CTA 1's half of B
+    is written by its own copies, whose completion has to be counted in CTA 0: the MMA that CTA 0 issues reads it."""
+    src = source("laph_tc.cu")
+    arrives = re.findall(r"mbarrier\.arrive[\w.:]*shared::cluster\.b64", src)
+    assert arrives and all(".release.cluster." in a or ".relaxed.cluster." in a for a in arrives)
+    k = body(src, "tc_pair_kernel(")
+    assert re.search(r"if \(rank\)\s*tma_b1\([^;]*peer_addr\(fb, 0\)\)", k)
+    # barriers that the other CTA's threads or MMAs arrive on are waited for at cluster scope
+    for bar in ("a_full", "acc_empty", "acc_full", "empty", "tempty"):
+        assert not re.search(r"warp_wait\(c, &S->%s\[" % bar, k), bar
