@@ -311,7 +311,10 @@ typedef struct {
     int tile_cols;   /* tensor-core modes: complex columns per tile: 104, 96, 80 or 64 in layout 0; 176 (default),
                         192, 208 or 128 in layout 1.  0 with layout 0: the plan takes the shape (either layout, or tiles
                         of 128 rows x 208 columns worked by pairs of CTAs) with the lowest estimated time, 104 or 96
-                        columns of layout 0 for small problems; every shape gives the same results */
+                        columns of layout 0 for small problems.  Every shape adds the same products over the
+                        same drains, and with one drain interval for all tiles GB300 gives the same bits for
+                        all of them; an interval of its own for tiles without meson rows (chunk_sites_b) applies
+                        to rows that depend on the shape, within the mode's error bound */
     int layout;      /* tensor-core modes: how the complex product is laid out on the real tensor cores.
                         0: every complex column of the phased operand is two real rows (re, im) of the
                         MMA's B operand, 128 complex rows per tile; 1: every complex row of the diquark / meson

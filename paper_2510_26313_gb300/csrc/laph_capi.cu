@@ -874,7 +874,11 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     // SHAPE_MARGIN: layout 1 has half the B-operand bytes and 64-row tiles
     // (meson rows alone fill half of a 128-row tile), a narrower tile of layout 0
     // may cover the columns in as many tiles, CTA pairs keep a stage ring of four
-    // buffers with many row vectors.  Every shape gives the same bits.
+    // buffers with many row vectors.  Every shape adds the same products over the
+    // same drains; within a k-step the layouts hand the products of imaginary parts
+    // over in exchanged slots, which changes no bit of the tensor core's sum (tested
+    // for all shapes).  Only with chunk_sites_b does a shape matter: it decides which
+    // rows share a tile with meson rows.
     if (tc && !opt_cols && !opt_layout) {
         const double us104 = shape_us(def.tile_cols, 0);
         if (laph::tc_ring_depth(p->max_staged, def.tile_cols, 0) < 4 &&
