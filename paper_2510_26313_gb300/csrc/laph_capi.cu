@@ -830,32 +830,47 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     // STAGE_US_COL per accumulator column (both layouts); whole tiles on the
     // first free CTA where there are few waves of them, else (or where the last
     // wave can be cut into drains) spread evenly.  A stage ring of fewer than
-    // four buffers costs RING_COST.
-    auto shape_us = [&](int nc, int r2) -> double {
+    // four buffers costs RING_COST.  `cut`: as if a thin last wave could always be
+    // cut; `real`: as this plan is, whose tiles stay whole where it has two drain
+    // intervals, one timeslice per chunk or too many extra partials.
+    struct ShapeUs {
+        double cut, real;
+    };
+    const bool per_ts = (flags & LAPH_PLAN_CHUNK_PER_TIMESLICE) && p->total_ts > 1;
+    auto shape_us = [&](int nc, int r2) -> ShapeUs {
         build_tiles(nc, r2);
         set_sum(def.sum_sites);
         const int ring = laph::tc_ring_depth(p->max_staged, nc, r2);
-        if (p->max_staged > laph::TC_MAX_STAGED || !ring) return 1e300;
-        double total = 0.0, bytes = 0.0;
-        long long n_tiles = 0;
+        if (p->max_staged > laph::TC_MAX_STAGED || !ring) return {1e300, 1e300};
         auto stage_us = [&](const TileDev &u) {
             const int n_real = r2 ? ((u.ncols + 15) & ~15) - u.cskip : 2 * ((u.ncols + 7) & ~7) - 2 * u.cskip;
             return r2 == 2 ? PAIR_STAGE_US + PAIR_STAGE_US_COL * n_real : STAGE_US + STAGE_US_COL * n_real;
         };
-        for (int n = 0; n < n_inst; n++) {
-            const InstDev &d = p->h_inst[n];
-            for (const TileDev &u : ones[n]) total += stage_us(u) * d.n_st * d.T;
-            n_tiles += (long long)ones[n].size() * d.n_sc * d.T;
-            bytes += (double)d.T * ((double)d.n_ct * d.n_st * laph::tc_stage_bytes(nc, r2) + 24.0 * d.Nc * d.V);
-        }
-        double us = total / workers();
-        if (n_tiles <= (long long)SPLIT_MAX_WAVES * workers()) {
-            std::vector<double> free_at(workers(), 0.0);
+        const int cs = drain_stages(), w = workers();
+        // the contraction of instances [n0, n1), all their timeslices or one of each
+        auto contraction = [&](int n0, int n1, bool one_t) -> ShapeUs {
+            double total = 0.0, extra = 0.0;   // extra: bytes of the partials when every unit is cut
+            long long n_tiles = 0, n_units = 0;
+            int st_max = 1;
+            for (int n = n0; n < n1; n++) {
+                const InstDev &d = p->h_inst[n];
+                const int T = one_t ? 1 : d.T;
+                for (const TileDev &u : ones[n]) total += stage_us(u) * d.n_st * T;
+                n_tiles += (long long)ones[n].size() * d.n_sc * T;
+                n_units += T;
+                for (int b0 = 0; b0 < d.n_st; b0 += d.sc_stages)
+                    extra += (double)T * ((std::min(d.sc_stages, d.n_st - b0) + cs - 1) / cs - 1) *
+                             (double)(d.n_outB + d.n_outM) * sizeof(float2);
+                st_max = std::max(st_max, d.sc_stages);
+            }
+            const double even = total / w;
+            if (n_tiles > (long long)SPLIT_MAX_WAVES * w) return {even, even};
+            std::vector<double> free_at(w, 0.0);
             const auto later = std::greater<double>();
             double end = 0.0;
-            for (int n = 0; n < n_inst; n++) {
+            for (int n = n0; n < n1; n++) {
                 const InstDev &d = p->h_inst[n];
-                for (int t = 0; t < d.T; t++)
+                for (int t = 0; t < (one_t ? 1 : d.T); t++)
                     for (const TileDev &u : ones[n])
                         for (int b0 = 0; b0 < d.n_st; b0 += d.sc_stages) {
                             std::pop_heap(free_at.begin(), free_at.end(), later);
@@ -864,9 +879,24 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
                             std::push_heap(free_at.begin(), free_at.end(), later);
                         }
             }
-            us = std::min(end, n_tiles >= 2 * workers() ? 1.04 * us : (1.0 + TILE_STAGES / 16.0) * us);
+            // two waves or more: one wave of tiles is cut; fewer: every unit
+            const bool many = n_tiles >= 2 * w;
+            const double us = std::min(end, (many ? 1.04 : 1.0 + (double)TILE_STAGES / std::min(cs, st_max)) * even);
+            if (many) extra *= std::min(1.0, (double)((w * n_units + n_tiles - 1) / n_tiles) / (double)n_units);
+            const bool whole = per_ts || (def.chunk_sites_b && def.chunk_sites_b != def.chunk_sites) ||
+                               extra > (double)SPLIT_MAX_BYTES;
+            return {us, whole ? end : us};
+        };
+        ShapeUs us = contraction(0, n_inst, false);
+        double bytes = 0.0;
+        if (per_ts) us.real = 0.0;
+        for (int n = 0; n < n_inst; n++) {
+            const InstDev &d = p->h_inst[n];
+            if (per_ts) us.real += d.T * contraction(n, n + 1, true).real;
+            bytes += (double)d.T * ((double)d.n_ct * d.n_st * laph::tc_stage_bytes(nc, r2) + 24.0 * d.Nc * d.V);
         }
-        return us * (ring < 4 ? RING_COST : 1.0) + bytes / (r2 ? PSI_BYTES_US_ROWS2 : PSI_BYTES_US);
+        const double f = ring < 4 ? RING_COST : 1.0, psi = bytes / (r2 ? PSI_BYTES_US_ROWS2 : PSI_BYTES_US);
+        return {us.cut * f + psi, us.real * f + psi};
     };
     // The default shape is 104 columns of layout 0, or 96 where the row vectors
     // a tile stages would leave its ring shallower than four buffers.  A plan
@@ -880,7 +910,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
     // for all shapes).  Only with chunk_sites_b does a shape matter: it decides which
     // rows share a tile with meson rows.
     if (tc && !opt_cols && !opt_layout) {
-        const double us104 = shape_us(def.tile_cols, 0);
+        const ShapeUs us104 = shape_us(def.tile_cols, 0);
         if (laph::tc_ring_depth(p->max_staged, def.tile_cols, 0) < 4 &&
             laph::tc_ring_depth(p->max_staged, 96, 0) > laph::tc_ring_depth(p->max_staged, def.tile_cols, 0))
             def.tile_cols = 96;
@@ -888,17 +918,29 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
         for (int n = 0; n < n_inst; n++)
             stages += (long long)ones[n].size() * p->h_inst[n].n_st * p->h_inst[n].T;
         // (a plan whose default tiles cannot stage their row vectors stays refused)
-        if (us104 < 1e300 && stages >= (long long)SHAPE_MIN_STAGES * sms) {
-            double best = (def.tile_cols == 96 ? shape_us(96, 0) : us104) * (1.0 - SHAPE_MARGIN);
-            const std::pair<int, int> shapes[] = {{96, 0}, {80, 0}, {64, 0}, {208, 1}, {176, 1}, {128, 1}, {laph::TC_PAIR_COLS, 2}};
-            for (const auto &sh : shapes) {
-                const double us = shape_us(sh.first, sh.second);
-                if (us < best) {
-                    best = us;
-                    def.tile_cols = sh.first;
-                    def.rows2 = sh.second;
-                }
-            }
+        if (us104.cut < 1e300 && stages >= (long long)SHAPE_MIN_STAGES * sms) {
+            const std::pair<int, int> shapes[] = {{def.tile_cols, 0}, {96, 0},  {80, 0},  {64, 0},
+                                                  {208, 1},           {176, 1}, {128, 1}, {laph::TC_PAIR_COLS, 2}};
+            constexpr int NSH = sizeof(shapes) / sizeof(shapes[0]);
+            ShapeUs us[NSH];
+            for (int k = 0; k < NSH; k++)
+                us[k] = k == 0 && def.tile_cols != 96 ? us104 : shape_us(shapes[k].first, shapes[k].second);
+            // the lowest estimate, if better than that of shape `best` by the margin
+            auto lowest = [&](int best, double ShapeUs::*e) {
+                double limit = us[best].*e * (1.0 - SHAPE_MARGIN);
+                for (int k = 0; k < NSH; k++)
+                    if (us[k].*e < limit) {
+                        best = k;
+                        limit = us[k].*e;
+                    }
+                return best;
+            };
+            // where the tiles stay whole, another shape than that of a plan whose last wave can be cut only if it is
+            // better by the margin again (L=18, N=40, 27 momenta, one timeslice, chunk_sites_b 192: 626 us with 35 tiles
+            // of 104 columns, 560 with 56 of 128 columns in layout 1; L=24, T=8, one timeslice per chunk 6850, 6320)
+            const std::pair<int, int> sh = shapes[lowest(lowest(0, &ShapeUs::cut), &ShapeUs::real)];
+            def.tile_cols = sh.first;
+            def.rows2 = sh.second;
         }
     }
     PCK(apply(def));
