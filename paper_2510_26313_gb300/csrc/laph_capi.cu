@@ -89,6 +89,9 @@ constexpr double SHAPE_MARGIN = 0.03;
 constexpr int SHAPE_MIN_STAGES = 16;   // per SM
 // Jobs of the B-operand pass per SM below which jobs are made shorter.
 constexpr int PSI_JOBS_PER_SM = 8;
+// Blocks of a scale or blocking launch that may find nothing to do (see
+// prep_runs): about 1 ns each, against a few microseconds for another launch.
+constexpr long long PREP_IDLE_BLOCKS = 4096;
 
 }  // namespace
 
@@ -150,6 +153,12 @@ struct laph_plan {
         long long n_red_split;   // blocks of their reduction
     };
     std::vector<Chunk> chunks;
+    // launches of the scale and blocking passes over the whole batch: consecutive units of similar size
+    struct PrepRun {
+        int unit0, n_units, nblk;   // nblk, elems: the most of any unit
+        long long elems;
+    };
+    std::vector<PrepRun> prep;
     // where units are cut into drains: the same schedule with whole site blocks,
     // for laph_plan_set_chunk_sites.  Its tiles and units follow the cut ones in
     // d_tiles, d_units and h_units (tile0 and unit0 count from the start of
@@ -277,6 +286,7 @@ static void free_plan(laph_plan *p)
 static int autotune(laph_plan *p, const laph::Sched &def,
                     const std::function<cudaError_t(const laph::Sched &)> &apply);
 static cudaError_t ensure_side(laph_plan *p);
+static std::vector<laph_plan::PrepRun> prep_runs(const laph_plan *p, int unit0, int n_units);
 
 static int tc_supported(int device)
 {
@@ -819,6 +829,7 @@ int laph_plan_create_opts(const laph_instance *inst, int n_inst, int mode, unsig
         const long long model = chunking(c.per_chunk == -2);   // also sets psi_target for several instances
         const long long pc = c.per_chunk >= 0 ? c.per_chunk : model;
         emit(pc, c.order);
+        if (tc) p->prep = prep_runs(p, 0, p->total_ts);
         p->sched = c;
         return upload();
     };
@@ -1117,21 +1128,50 @@ static int launch_tc_chunk(laph_plan *p, char *ws, size_t ci, const laph::TcConf
     return LAPH_OK;
 }
 
-// Scale and site-blocked copy of the units [unit0, unit0 + n_units): one launch each.
-static int launch_prep(laph_plan *p, char *ws, int unit0, int n_units, cudaStream_t s)
+// The units [unit0, unit0 + n_units) in runs that share a scale and a blocking
+// launch.  A launch has as many blocks per unit as the largest of its units
+// needs, so a run ends where the blocks without work would outnumber the others
+// (and PREP_IDLE_BLOCKS): units come in decreasing order of work, so these are few
+// runs.  One launch for L=4 timeslices beside a single L=48 one is 13,824 blocks
+// for each of them, 8 of which have work (5000 of them, N=8: 36.5 -> 1.0 ms an execute; one L=24 and
+// 300 L=8 timeslices, N=16: 578 -> 302 us).
+static std::vector<laph_plan::PrepRun> prep_runs(const laph_plan *p, int unit0, int n_units)
+{
+    std::vector<laph_plan::PrepRun> runs;
+    long long need = 0;
+    for (int u = unit0; u < unit0 + n_units; u++) {
+        const int n = p->h_units[u].inst, nb = p->h_inst[n].nblk;
+        const long long elems = p->phi_elems[n] / p->h_T[n];
+        if (!runs.empty()) {
+            laph_plan::PrepRun &r = runs.back();
+            const int most = std::max(r.nblk, nb);
+            const long long all = (long long)most * (r.n_units + 1);
+            if (all - (need + nb) <= std::max(need + nb, PREP_IDLE_BLOCKS)) {
+                need += nb;
+                r.n_units++;
+                r.nblk = most;
+                r.elems = std::max(r.elems, elems);
+                continue;
+            }
+        }
+        need = nb;
+        runs.push_back({u, 1, nb, elems});
+    }
+    return runs;
+}
+
+// Scale and site-blocked copy of the units of these runs.
+static int launch_prep(laph_plan *p, char *ws, const std::vector<laph_plan::PrepRun> &runs, cudaStream_t s)
 {
     unsigned *maxbits = (unsigned *)(ws + p->off_maxbits);
-    long long elems = 1;
-    int nblk = 1;
-    for (int n = 0; n < p->n_inst; n++) {
-        elems = std::max(elems, p->phi_elems[n] / p->h_T[n]);
-        nblk = std::max(nblk, p->h_inst[n].nblk);
-    }
     const InstDev &d = p->h_inst[0];   // the kind of instance is the plan's
-    cudaError_t e = laph::launch_scale_max(p->d_inst, p->d_units + unit0, n_units, d.n_fields, elems, maxbits, s);
-    if (e != cudaSuccess) return cuda_fail(e, "scale_max");
-    e = laph::launch_blockify(p->d_inst, p->d_units + unit0, n_units, nblk, d.kind == laph::INST_TRIPLETS, maxbits, s);
-    if (e != cudaSuccess) return cuda_fail(e, "blockify");
+    for (const laph_plan::PrepRun &r : runs) {
+        const laph::PsiUnit *units = p->d_units + r.unit0;
+        cudaError_t e = laph::launch_scale_max(p->d_inst, units, r.n_units, d.n_fields, r.elems, maxbits, s);
+        if (e != cudaSuccess) return cuda_fail(e, "scale_max");
+        e = laph::launch_blockify(p->d_inst, units, r.n_units, r.nblk, d.kind == laph::INST_TRIPLETS, maxbits, s);
+        if (e != cudaSuccess) return cuda_fail(e, "blockify");
+    }
     return LAPH_OK;
 }
 
@@ -1144,7 +1184,7 @@ static int launch_batch(laph_plan *p, void *workspace, cudaStream_t s, bool clea
         if (!workspace || ((uintptr_t)workspace) % 256) return LAPH_ERR_WORKSPACE;
         char *ws = (char *)workspace;
         if (!cleared) CK(cudaMemsetAsync(ws, 0, p->ws_zero_bytes, s));
-        const int rc = launch_prep(p, ws, 0, p->total_ts, s);
+        const int rc = launch_prep(p, ws, p->prep, s);
         if (rc != LAPH_OK) return rc;
         const laph::TcConfig cfg = tc_config(p);
         for (size_t ci = 0; ci < p->chunks.size(); ci++) {
@@ -1531,9 +1571,10 @@ int laph_plan_launches_per_execute(const laph_plan *plan, int *n)
 {
     if (!plan || !n) return LAPH_ERR_ARG;
     const int ptr_launches = (plan->n_inst + 63) / 64;
+    int prep = 0;   // scale, blockify
+    for (const laph_plan::PrepRun &r : plan->prep) prep += 2 * ((r.n_units + 65534) / 65535);
     if (is_tc_mode(plan->mode))
-        *n = ptr_launches + 2 * ((plan->total_ts + 65534) / 65535) /* scale, blockify */ +
-             3 * (int)plan->chunks.size() /* psi, contraction, FP64 site reduction */ +
+        *n = ptr_launches + prep + 3 * (int)plan->chunks.size() /* psi, contraction, FP64 site reduction */ +
              (!plan->chunks.empty() && plan->chunks.back().n_split > 0 &&
               plan->chunks.back().n_split < plan->chunks.back().n_units) /* a reduction for either kind of unit */;
     else
@@ -1683,7 +1724,7 @@ static int execute_host_body(laph_plan *plan, const void *const *phi_host, void 
     for (size_t ci = 0; ci < nc; ci++) {
         const laph_plan::Chunk &c = plan->chunks[ci];
         CK(cudaStreamWaitEvent(s, plan->ev_in[ci], 0));
-        int rc = launch_prep(plan, ws, c.unit0, c.n_units, s);
+        int rc = launch_prep(plan, ws, prep_runs(plan, c.unit0, c.n_units), s);
         if (rc == LAPH_OK) rc = launch_tc_chunk(plan, ws, ci, cfg, s);
         if (rc != LAPH_OK) return rc;
         // the outputs of chunk ci are final once its site reduction (side stream) is done

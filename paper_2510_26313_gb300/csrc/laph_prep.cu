@@ -181,9 +181,10 @@ cudaError_t launch_diff_norms(const void *a, bool a_c64, const double2 *b, long 
 // order like their bit patterns).  The tensor-core kernel turns it into an
 // exact power-of-two rescale before splitting into hi/lo halves.
 //
-// One launch covers every (instance, timeslice) of the units given (and every
-// field): block (x, u, field) of unit u, grid-strided in x.  A ragged batch of
-// 24 instances took a launch of a few microseconds for each of them before.
+// One launch covers all (instance, timeslice) units given (and every field):
+// block (x, u, field) of unit u, grid-strided in x.  A ragged batch of 24
+// instances took a launch of a few microseconds for each of them before.  The
+// caller gives units of similar size: the grid has the largest unit's blocks.
 __global__ void __launch_bounds__(256) scale_max_kernel(const InstDev *__restrict__ d_inst,
                                                         const PsiUnit *__restrict__ units, unsigned *__restrict__ maxbits)
 {
