@@ -393,7 +393,8 @@ def lanczos(U, L: int, n_ev: int, n_krylov: int, cheb_degree: int = 0, cheb_lo: 
     residual norms float64 [T][n_ev] as numpy arrays).  workspace: a uint8 CUDA tensor of
     lanczos_workspace_size bytes (None: the call allocates its own).  stats: a dict that receives
     the call's event-timed breakdown (total_ms, setup_ms, apply_ms, orth_ms, ritz_ms, launches,
-    apply_launches)."""
+    apply_launches).  pdl has no effect any more: filter steps are always programmatic dependents of
+    their predecessors."""
     import torch
     T = _check_links(U, L)
     if out is None:

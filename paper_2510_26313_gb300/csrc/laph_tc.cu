@@ -1587,7 +1587,7 @@ __device__ __forceinline__ void red_store(const InstDev &I, int t, long long e, 
 // way.  The additions of one entry are a serial chain, so a thread takes one
 // entry (more blocks in flight) and issues RED_BATCH loads ahead of it: small
 // outputs are bound by load latency (L=24, N=32, 7 momenta, one timeslice:
-// 41,720 entries x 108 drains, 36 MB, read by 163 blocks).
+// 41,888 entries x 108 drains, 36 MB, read by 164 blocks).
 constexpr int RED_THREADS = 256;
 constexpr int RED_PER_THREAD = TC_RED_BLOCK / RED_THREADS;
 constexpr int RED_BATCH = 16;
