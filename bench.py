@@ -42,13 +42,13 @@ WORKLOADS = {
 METRIC = "baryon+meson block complex TFLOP/s at L=32,N=64,Np=19; tensor-pipe %; rel err vs FP64"
 
 # DRAM bytes (read + write) of tc_kernel per byte of B-operand stage images it consumes, from the ncu captures
-# summarised in profiles/, by (tile rows, tile columns): tc_kernel_L24_T2_N64_P19_full.md (1.941 GB for 2 x 12 x 1728
-# stage images of 39,936 B, tc_kernel<0,3,104,0>) and tc_kernel_rowdoubled208_L24_T2_N64_P19_full.md (1.071 GB for
+# summarised in profiles/, by (tile rows, tile columns): tc_kernel_L24_T2_N64_P19_full.md (2.027 GB for 2 x 12 x 1728
+# stage images of 39,936 B, tc_kernel<0,3,104,0>) and tc_kernel_rowdoubled208_L24_T2_N64_P19_full.md (1.082 GB for
 # 2 x 6 x 1728 images of 39,936 B, tc_kernel<0,3,208,1>).  The contraction's DRAM traffic is dominated by those images,
 # so a launch's traffic is the ratio times its image bytes; a plan of another tile shape reports no traffic.  To be
 # retaken whenever the kernel changes.
-TC_DRAM_PER_IMAGE_BYTE = {(128, 104): 1.941e9 / (2 * 12 * 1728 * 39936),
-                          (64, 208): 1.071e9 / (2 * 6 * 1728 * 39936)}
+TC_DRAM_PER_IMAGE_BYTE = {(128, 104): 2.027e9 / (2 * 12 * 1728 * 39936),
+                          (64, 208): 1.082e9 / (2 * 6 * 1728 * 39936)}
 TC_PROFILE = {(128, 104): "profiles/tc_kernel_L24_T2_N64_P19_full.md",
               (64, 208): "profiles/tc_kernel_rowdoubled208_L24_T2_N64_P19_full.md"}
 
@@ -560,7 +560,7 @@ LANCZOS = {
 # DRAM bytes (read + write) of one lap_soa_kernel launch on a group of 8 timeslices at L=32 with links read as three
 # rows, from the ncu capture summarised in profiles/lap_soa_kernel_L32_T8_group8_full.md (warm L2, the launch shape of
 # every filter launch of the L=32, T=64 workload); to be retaken whenever the kernel changes
-LAP_SOA_TRAFFIC = 12.7e6
+LAP_SOA_TRAFFIC = 12.0e6
 
 
 def laplacian_bytes_per_site(with_z: bool, link_rows: int = 3) -> int:
